@@ -1,6 +1,6 @@
 // Hand-written BF16 GEMM on the 5th-generation tensor cores (tcgen05):
 //   C[M x N] = A[M x K] . B[N x K]^T   (both operands K-major in shared memory),
-// FP32 accumulation in tensor memory (TMEM), fused epilogues.  One CTA of 128
+// FP32 accumulation in tensor memory (TMEM).  One CTA of 128
 // threads owns a 128 x BN tile (BN <= 256, multiple of 16); operands are staged
 // by all threads into the canonical no-swizzle K-major layout (8-row x 16-byte
 // core matrices) in two shared-memory stages, one elected thread issues
@@ -23,13 +23,6 @@ constexpr int SMEM = 2 * (A_STAGE + B_STAGE) + 64;
 constexpr int TMEM_COLS = 256;
 constexpr long long WAIT_LIMIT = 1ll << 24;  // try_wait polls before declaring a timeout
 
-enum Epi {
-    EPI_F32 = 0,        // C (fp32) = acc             (atomicAdd when split over K)
-    EPI_BIAS_SILU = 1,  // Z = acc + bias (bf16), H = silu(Z) (bf16)
-    EPI_BIAS = 2,       // C (fp32) = acc + bias
-    EPI_DSILU = 3       // dZ = acc * silu'(Zin) (bf16)
-};
-
 struct GemmArgs {
     const __nv_bfloat16 *A;
     long long lda;      // A(m,k) = A[m*lda + k], or A[k*lda + m] when transposed
@@ -38,14 +31,8 @@ struct GemmArgs {
     int M, N, K;        // K multiple of 16
     int BN;             // N-tile (multiple of 16, <= 256)
     int kper;           // K range per blockIdx.z (multiple of 64), split-K
-    int epi;
-    float *C;
+    float *C;           // fp32, atomically added when split over K
     long long ldc;
-    const float *bias;
-    __nv_bfloat16 *Z, *H;
-    const __nv_bfloat16 *Zin;
-    __nv_bfloat16 *dZ;
-    long long ldz;
     int *err;           // set to 1 on a bounded-wait timeout
 };
 
@@ -71,13 +58,6 @@ __host__ __device__ __forceinline__ uint32_t make_idesc(int M, int N)
            | (1u << 10)                    // B format BF16
            | ((uint32_t)(N >> 3) << 17)    // N / 8
            | ((uint32_t)(M >> 4) << 24);   // M / 16
-}
-
-__device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
-__device__ __forceinline__ float dsilu(float z)
-{
-    float s = 1.f / (1.f + __expf(-z));
-    return s * (1.f + z * (1.f - s));
 }
 
 // Wait for the phase of `parity` of the mbarrier to complete, polling at most
@@ -257,28 +237,11 @@ __global__ void __launch_bounds__(128, 1) gemm_bf16(GemmArgs g)
                 const int n = nb + i;
                 if (n >= g.N) break;
                 float a = __uint_as_float(v[i]);
-                const long long off = (long long)row * g.ldz + n;
-                switch (g.epi) {
-                case EPI_F32:
-                    if (gridDim.z > 1)
-                        atomicAdd(g.C + (long long)row * g.ldc + n, a);
-                    else
-                        g.C[(long long)row * g.ldc + n] = a;
-                    break;
-                case EPI_BIAS:
-                    g.C[(long long)row * g.ldc + n] = a + g.bias[n];
-                    break;
-                case EPI_BIAS_SILU: {
-                    float z = a + g.bias[n];
-                    __nv_bfloat16 zb = __float2bfloat16(z);
-                    g.Z[off] = zb;
-                    g.H[off] = __float2bfloat16(silu(__bfloat162float(zb)));
-                    break;
-                }
-                case EPI_DSILU:
-                    g.dZ[off] = __float2bfloat16(a * dsilu(__bfloat162float(g.Zin[off])));
-                    break;
-                }
+                float *c = g.C + (long long)row * g.ldc + n;
+                if (gridDim.z > 1)
+                    atomicAdd(c, a);
+                else
+                    *c = a;
             }
         }
     }
