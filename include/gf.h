@@ -178,10 +178,13 @@ size_t gf_grid_bytes(gf_plan_t plan);
  *             GF_OUT_GRAD and GF_OUT_HESSDIFF (GF_DERIV2D plans; the latter with k2 > 0)
  *   dev_out   n * entries complex values, [n][entries], device memory
  * The plan is not modified by an evaluation: each call takes its scratch (the
- * far- and near-branch target lists, 12 bytes per target plus 4 KiB; for 3D
- * plans also about 2.3 bytes per target of far-list counts and tickets and the
- * far sums' slab partials, 4 * entries * (8 or 16) bytes per target for float or
- * double plans) from the library's stream-ordered memory pool on cuda_stream
+ * far- and near-branch target lists, 12 bytes per target plus 9 KiB; for 3D
+ * plans also about 8 bytes per target (4 MiB at most) of far-list counts and
+ * tickets, the far sums' slab partials, 4 * entries * (8 or 16) bytes per target
+ * for float or double plans (up to 16 times that below 16384 targets), and, from
+ * 12288 to 327680 targets on (by precision and kind), the far weights' images:
+ * 61 MB (double) or 10 MB (float) per entry) from the library's stream-ordered
+ * memory pool on cuda_stream
  * and returns it in stream order, so calls on one plan may run concurrently on
  * different streams and threads.  Results are reproducible: the same plan and
  * targets give the same bits at every call (the far targets are grouped by a

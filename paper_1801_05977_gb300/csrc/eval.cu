@@ -145,6 +145,7 @@ __device__ __forceinline__ void far_deposit(const EvalArgs &a, int kind, int w, 
     for (int e = 0; e < NE; ++e) {
         if (e >= ne) break;
         C sum = __ldcg(buf + slot * ne + e);
+#pragma unroll 4
         for (int s = 1; s < nslab; ++s) sum = cadd(sum, __ldcg(buf + ((size_t)s * nslot + slot) * ne + e));
         add_c(o + e, sum);
     }
@@ -795,15 +796,18 @@ __device__ void far_scatter_body(const EvalArgs &a, int blk, int nblk, int *off)
 // bit for bit.  Three passes over segments of a.segsize targets, one warp each:
 // counts per segment and bucket, their exclusive scan over the segments (per
 // bucket, from the bucket's start), and the scatter in index order.
-__global__ void __launch_bounds__(256) far_seg_count(EvalArgs a)
+constexpr int SEG_WARPS = 4;
+
+__global__ void __launch_bounds__(32 * SEG_WARPS) far_seg_count(EvalArgs a)
 {
-    __shared__ int h[8][GF_FAR_BUCKETS];
+    __shared__ int h[SEG_WARPS][GF_FAR_BUCKETS];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int seg = blockIdx.x * 8 + w;
+    const int seg = blockIdx.x * SEG_WARPS + w;
     if (seg >= a.nseg) return;
     for (int b = lane; b < GF_FAR_BUCKETS; b += 32) h[w][b] = 0;
     __syncwarp();
     const int64_t i0 = (int64_t)seg * a.segsize, i1 = min(i0 + (int64_t)a.segsize, a.n);
+#pragma unroll 4
     for (int64_t i = i0 + lane; i < i1; i += 32) {
         const int c = a.far_idx[i];
         if (c >= 0) atomicAdd(&h[w][c], 1);
@@ -843,29 +847,39 @@ __global__ void __launch_bounds__(1024) far_seg_scan(EvalArgs a)
 
 // Each warp walks its segment in index order, 32 targets a step: the lanes with
 // the same bucket take consecutive positions from the segment's running start.
-__global__ void __launch_bounds__(256) far_seg_scatter(EvalArgs a)
+__global__ void __launch_bounds__(32 * SEG_WARPS) far_seg_scatter(EvalArgs a)
 {
-    __shared__ int pos0[8][GF_FAR_BUCKETS];
+    __shared__ int pos0[SEG_WARPS][GF_FAR_BUCKETS];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int seg = blockIdx.x * 8 + w;
+    const int seg = blockIdx.x * SEG_WARPS + w;
     if (seg >= a.nseg) return;
     const int *src = a.seghist + (size_t)seg * GF_FAR_BUCKETS;
     for (int b = lane; b < GF_FAR_BUCKETS; b += 32) pos0[w][b] = src[b];
     __syncwarp();
     const unsigned below = (1u << lane) - 1u;
     const int64_t i0 = (int64_t)seg * a.segsize, i1 = min(i0 + (int64_t)a.segsize, a.n);
-    for (int64_t j = i0; j < i1; j += 32) {
-        const int64_t i = j + lane;
-        const int c = i < i1 ? a.far_idx[i] : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, c);
-        const int before = __popc(peers & below);
-        const int pos = c >= 0 ? pos0[w][c] + before : 0;
-        __syncwarp();
-        if (c >= 0) {
-            a.far_sorted[pos] = (int)i;
-            if (before == 0) pos0[w][c] += __popc(peers);
+    // eight steps' codes are loaded at once
+    for (int64_t j0 = i0; j0 < i1; j0 += 256) {
+        int code[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int64_t i = j0 + 32 * u + lane;
+            code[u] = i < i1 ? a.far_idx[i] : -1;
         }
-        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int c = code[u];
+            if (__ballot_sync(0xffffffffu, c >= 0) == 0u) continue;
+            const unsigned peers = __match_any_sync(0xffffffffu, c);
+            const int before = __popc(peers & below);
+            const int pos = c >= 0 ? pos0[w][c] + before : 0;
+            __syncwarp();
+            if (c >= 0) {
+                a.far_sorted[pos] = (int)(j0 + 32 * u + lane);
+                if (before == 0) pos0[w][c] += __popc(peers);
+            }
+            __syncwarp();
+        }
     }
 }
 
@@ -917,8 +931,13 @@ __device__ __forceinline__ void set_entry(BetaEntryF &e, double b, double ib)
 // of propagating indices in row-major order of the sub-box pbox = [n1lo, n1hi,
 // n2lo, n2hi] (ballot compaction keeps the order fixed).
 template <typename E>
-__global__ void series_tables(EvalArgs a, E *tab, double2 *exptab, PropEntry *prop, int *nprop, int4 pbox)
+__global__ void series_tables(EvalArgs a, E *tab, double2 *exptab, longlong2 *trig, PropEntry *prop, int *nprop, int4 pbox)
 {
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < GF_TRIG_STEPS; j += gridDim.x * blockDim.x) {
+        double sn, cn;
+        sincospi(2.0 * j / GF_TRIG_STEPS, &sn, &cn);
+        trig[j] = longlong2{__double2ll_rn(cn * 0x1p61), __double2ll_rn(sn * 0x1p61)};
+    }
     const int W2 = a.n2hi - a.n2lo + 1;
     const int tot = (a.n1hi - a.n1lo + 1) * W2;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += gridDim.x * blockDim.x) {
@@ -1992,14 +2011,73 @@ __device__ __forceinline__ int far_take(int *counter, int nitems)
     return t < nitems ? t : -1;
 }
 
+// Row slabs per chunk at most.  A short list leaves the GPU empty unless its chunks are cut
+// into single rows (1017 targets: far3d_f64 378 us with 8 slabs, 90 us with 32); from about
+// 300 chunks on the slabs' repeated set-up costs more (13000 far targets: 559 us for
+// the evaluation with 8 slabs, 681 us with 32).  The float sums' set-up is cheap.
+constexpr int FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_LONG = 300;
+
+// Chunks of a far launch: all of the list, or those of the cells that the product
+// path left over (a.rej: their number, tiles per cell, a flag per cell).  The t-th
+// chunk taken from the end of the list is `at(t)`, -1 where the last cell ends
+// short of its tiles.  Called by all threads of the block.
+struct FarChunks {
+    int nch, count, per;
+    const short *cell;
+    __device__ __forceinline__ FarChunks(const EvalArgs &a, short *list)
+    {
+        count = a.far_count[0];
+        nch = (count + 31) >> 5;
+        per = 0;
+        cell = nullptr;
+        if (a.rej) {
+            per = 4 * a.rej[1];
+            const int nrej = a.rej[0], ncell = (nch + per - 1) / per;
+            if (nrej > 0) {
+                // the flagged cells in order, by one warp
+                if (threadIdx.x < 32) {
+                    int n = 0;
+                    for (int c0 = 0; c0 < ncell; c0 += 32) {
+                        const int c = c0 + (int)threadIdx.x;
+                        const bool f = c < ncell && a.rej[2 + c] != 0;
+                        const unsigned bal = __ballot_sync(0xffffffffu, f);
+                        if (f) list[n + __popc(bal & ((1u << threadIdx.x) - 1u))] = (short)c;
+                        n += __popc(bal);
+                    }
+                }
+                __syncthreads();
+            }
+            nch = nrej * per;
+            cell = list;
+        }
+    }
+    __device__ __forceinline__ int at(int t) const
+    {
+        const int w = nch - 1 - t;
+        if (!cell) return w;
+        const int c = cell[w / per] * per + w % per;
+        return c * 32 < count ? c : -1;
+    }
+    // row slabs per chunk: by the chunks of this launch, capped by the scratch of the whole list
+    __device__ __forceinline__ int slabs(const EvalArgs &a, int kind, bool fp64) const
+    {
+        const int smax = !fp64 ? FAR_SLABS_MAX / 2 : nch <= FAR_LONG ? FAR_SLABS_MAX : FAR_SLABS_LONG;
+        return far_slabs_capped(a, kind, (count + 31) >> 5, far_slabs(nch, smax));
+    }
+};
+static_assert(GF_FAR_CELLS < 32768, "cells are listed as short");
+
 template <int NF, bool TAILS>
 __global__ void __launch_bounds__(128, NF == 1 ? 5 : 1) far3d_f64(EvalArgs a)
 {
-    const int count = a.far_count[0];
-    const int nch = (count + 31) >> 5, S = far_slabs_capped(a, 0, nch, far_slabs(nch, 8));
+    __shared__ short rejected[GF_FAR_CELLS];
+    const FarChunks ch(a, rejected);
+    const int S = ch.slabs(a, 0, true);
     int *ctr = a.far_count + GF_WORK_SLOT;
-    for (int t = far_take(ctr, nch * S); t >= 0; t = far_take(ctr, nch * S))
-        far3d_f64_chunk<NF, TAILS>(a, nch - 1 - t / S, count, t % S, S);
+    for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
+        const int w = ch.at(t / S);
+        if (w >= 0) far3d_f64_chunk<NF, TAILS>(a, w, ch.count, t % S, S);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2092,11 +2170,14 @@ __device__ void far3d_tail_chunk(const EvalArgs &a, int w, int count, int slab, 
 template <int NF>
 __global__ void __launch_bounds__(128) far3d_tail(EvalArgs a)
 {
-    const int count = a.far_count[0];
-    const int nch = (count + 31) >> 5, S = far_slabs_capped(a, 1, nch, far_slabs(nch, 8));
+    __shared__ short rejected[GF_FAR_CELLS];
+    const FarChunks ch(a, rejected);
+    const int S = ch.slabs(a, 1, true);
     int *ctr = a.far_count + GF_TAIL_SLOT;
-    for (int t = far_take(ctr, nch * S); t >= 0; t = far_take(ctr, nch * S))
-        far3d_tail_chunk<NF>(a, nch - 1 - t / S, count, t % S, S);
+    for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
+        const int w = ch.at(t / S);
+        if (w >= 0) far3d_tail_chunk<NF>(a, w, ch.count, t % S, S);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2269,11 +2350,14 @@ __device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, i
 template <int NF>
 __global__ void __launch_bounds__(128) far3d_f32(EvalArgs a)
 {
-    const int count = a.far_count[0];
-    const int nch = (count + 31) >> 5, S = far_slabs_capped(a, 0, nch, far_slabs(nch, 4));
+    __shared__ short rejected[GF_FAR_CELLS];
+    const FarChunks ch(a, rejected);
+    const int S = ch.slabs(a, 0, false);
     int *ctr = a.far_count + GF_WORK_SLOT;
-    for (int t = far_take(ctr, nch * S); t >= 0; t = far_take(ctr, nch * S))
-        far3d_f32_chunk<NF>(a, nch - 1 - t / S, count, t % S, S);
+    for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
+        const int w = ch.at(t / S);
+        if (w >= 0) far3d_f32_chunk<NF>(a, w, ch.count, t % S, S);
+    }
 }
 
 // Batched far kernel: one persistent launch for all pairs.  The work items of
@@ -2495,18 +2579,19 @@ cudaError_t launch_far_f64(const EvalArgs &a, int nsm, cudaStream_t s, const Eva
 void launch_far_list(const EvalArgs &a, int nsm, cudaStream_t s)
 {
     if (a.seghist) {
-        const int blocks = (a.nseg + 7) / 8;
-        far_seg_count<<<blocks, 256, 0, s>>>(a);
+        const int blocks = (a.nseg + SEG_WARPS - 1) / SEG_WARPS;
+        far_seg_count<<<blocks, 32 * SEG_WARPS, 0, s>>>(a);
         far_seg_scan<<<GF_FAR_BUCKETS / 32, 1024, 0, s>>>(a);
-        far_seg_scatter<<<blocks, 256, 0, s>>>(a);
+        far_seg_scatter<<<blocks, 32 * SEG_WARPS, 0, s>>>(a);
     } else {
         far_scatter<<<nsm * 2, 256, 0, s>>>(a);
     }
 }
 
 template <typename R>
-cudaError_t launch_eval_t(const EvalArgs &a, cudaStream_t s, cudaEvent_t ev_mid, const EvalFork *fork)
+cudaError_t launch_eval_t(const EvalArgs &a0, cudaStream_t s, cudaEvent_t ev_mid, const EvalFork *fork)
 {
+    EvalArgs a = a0;
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -2537,6 +2622,10 @@ cudaError_t launch_eval_t(const EvalArgs &a, cudaStream_t s, cudaEvent_t ev_mid,
         }
         if (ev_mid) cudaEventRecord(ev_mid, s);
         launch_far_list(a, nsm, s);
+        if (a.mma) {
+            cudaError_t e = gf_launch_far_product(a, sizeof(R) == 8 ? GF_FP64 : GF_FP32_SPLIT, nsm, s);
+            if (e != cudaSuccess) return e;
+        }
         if (sizeof(R) == 8) {
             cudaError_t e = launch_far_f64<1>(a, nsm, s, fork);
             if (e != cudaSuccess) return e;
@@ -2551,6 +2640,10 @@ cudaError_t launch_eval_t(const EvalArgs &a, cudaStream_t s, cudaEvent_t ev_mid,
         }
         if (ev_mid) cudaEventRecord(ev_mid, s);
         launch_far_list(a, nsm, s);
+        if (a.mma) {
+            cudaError_t e = gf_launch_far_product(a, sizeof(R) == 8 ? GF_FP64 : GF_FP32_SPLIT, nsm, s);
+            if (e != cudaSuccess) return e;
+        }
         if (sizeof(R) == 8) {
             cudaError_t e = launch_far_f64<7>(a, nsm, s, fork);
             if (e != cudaSuccess) return e;
@@ -2599,14 +2692,14 @@ cudaError_t gf_launch_eval_batch(const EvalBatch &b, int precision, cudaStream_t
     return precision == GF_FP64 ? launch_eval_batch_t<double>(b, s) : launch_eval_batch_t<float>(b, s);
 }
 
-cudaError_t gf_launch_series_tables(const EvalArgs &a, int precision, double2 *exptab, PropEntry *prop, int *nprop,
+cudaError_t gf_launch_series_tables(const EvalArgs &a, int precision, double2 *exptab, longlong2 *trig, PropEntry *prop, int *nprop,
                                     const int pbox[4], cudaStream_t s)
 {
     const int4 pb = make_int4(pbox[0], pbox[1], pbox[2], pbox[3]);
     if (precision == GF_FP64)
-        series_tables<BetaEntry><<<256, 256, 0, s>>>(a, (BetaEntry *)const_cast<void *>(a.btab), exptab, prop, nprop, pb);
+        series_tables<BetaEntry><<<256, 256, 0, s>>>(a, (BetaEntry *)const_cast<void *>(a.btab), exptab, trig, prop, nprop, pb);
     else
-        series_tables<BetaEntryF><<<256, 256, 0, s>>>(a, (BetaEntryF *)const_cast<void *>(a.btab), exptab, prop, nprop, pb);
+        series_tables<BetaEntryF><<<256, 256, 0, s>>>(a, (BetaEntryF *)const_cast<void *>(a.btab), exptab, trig, prop, nprop, pb);
     gf_count_launch(1);
     return cudaGetLastError();
 }

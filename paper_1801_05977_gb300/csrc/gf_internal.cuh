@@ -221,7 +221,34 @@ struct EvalArgs {
                             // followed by exptab_n float4 (hi, lo of e^{-y_j}, y_j, 0)
     int exptab_n, exptab_j0;
     double bmin;            // smallest |beta_n| over the evanescent n (this value or a larger one, never smaller)
+    double bprop;           // smallest beta_n over the propagating n (0: there are none)
+    // far series by matrix products (3D; null: by the series kernels alone): scratch of
+    // mma_cells cells; rej: cells left to the series kernels (their number, 128-target
+    // tiles per cell, the cells), null: every far target is theirs
+    void *mma;
+    int mma_cells;
+    const longlong2 *trig;  // e^{2 pi i j/GF_TRIG_STEPS}, 2^61 for 1
+    const int *rej;
+    int *err;               // device error word of the plan (bounded waits)
 };
+
+#define GF_TRIG_STEPS 1024
+// Cells of the product path per evaluation: enough that a cell is narrow in |x3| (its
+// expansion short), few enough that their weights cost little.
+#ifndef GF_FAR_CELLS
+#define GF_FAR_CELLS 152
+#endif
+// Targets from which an evaluation takes the product path (uniform targets, |x3| <= 1, times of
+// the whole evaluation, series kernels against products): double Helmholtz 263 / 418 us at 8000
+// (there the cells are too wide in |x3|), 408 / 286 at 16000; double Maxwell 1090 / 1312 at 16000,
+// 1832 / 967 at 32000; split Helmholtz 193 / 216 at 128000, 297 / 277 at 256000; split Maxwell
+// 704 / 714 at 256000, 1264 / 1150 at 512000.
+inline int64_t gf_far_product_min(int precision, int nf)
+{
+    return precision == GF_FP64 ? (nf == 1 ? 12288 : 20480) : (nf == 1 ? 196608 : 327680);
+}
+size_t gf_far_product_bytes(int precision, int64_t n, int nent, int *maxcells);
+cudaError_t gf_launch_far_product(EvalArgs &a, int precision, int nsm, cudaStream_t s);
 
 // Entries per unit of y of the far kernel's exponential table e^{-y_j}
 // (a power of two from 128 to 4096).
@@ -231,7 +258,7 @@ struct EvalArgs {
 
 // Far targets are bucketed by b = floor(NB c / |x_last|) (clamped to NB-1) so
 // that the lanes of a warp share nearly the same series truncation radius.
-#define GF_FAR_BUCKETS 256
+#define GF_FAR_BUCKETS 1024
 // scratch counters: [0] far count, [1..NB] bucket sizes, [NB+1..2NB] cursors,
 // [GF_WORK_SLOT] far work items handed out so far, [GF_TAIL_SLOT] the same for
 // the float-tail kernel of double-precision plans, [GF_NEAR_SLOT] length of the
@@ -275,7 +302,7 @@ cudaError_t gf_launch_cheb_deriv(const double *rr, const double *wy, int Q2, int
                                  cudaStream_t s);
 cudaError_t gf_launch_synth_batch(const SynthBatch &b, int precision, cudaStream_t s);
 cudaError_t gf_launch_eval_batch(const EvalBatch &b, int precision, cudaStream_t s);
-cudaError_t gf_launch_series_tables(const EvalArgs &a, int precision, double2 *exptab, PropEntry *prop, int *nprop,
+cudaError_t gf_launch_series_tables(const EvalArgs &a, int precision, double2 *exptab, longlong2 *trig, PropEntry *prop, int *nprop,
                                     const int pbox[4], cudaStream_t s);
 cudaError_t gf_launch_e_table(const double *tt, int Q, int Mlast, double qs, double2 *E, float2 *Ef, cudaStream_t s);
 // far-region grid: the planes' coefficients into a.work ([nf][L3count][M2][M1], FFT

@@ -127,9 +127,11 @@ struct gf_plan_s {
     PropEntry *prop = nullptr;        // propagating indices, then their count
     int *nprop_dev = nullptr;
     cudaStream_t stream = nullptr;    // stream of the plan's creation
+    longlong2 *trig = nullptr;        // e^{2 pi i j/GF_TRIG_STEPS} (3D)
     double2 *exptab = nullptr;        // (e^{-y_j}, y_j), y_j = (j - exptab_j0)/GF_EXPTAB_STEPS, then a float4 copy
     int exptab_n = 0, exptab_j0 = 0;
     double bmin_ev = 1e300;           // smallest evanescent |beta_n|
+    double bmin_prop = 0.0;           // smallest propagating beta_n (0: none)
     int n1lo = 0, n1hi = -1, n2lo = 0, n2hi = -1;
     SynthArgs sa{};
     // Launch lock: serialises the host-side enqueue of concurrent calls on this
@@ -259,7 +261,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     const double a1 = alpha[0], a2 = dim == 3 ? alpha[1] : 0.0;
 
     // Wood anomaly (Sec. 1): beta_n = 0 for some n.  Only |alpha_n| ~ k matters.
-    double bmin_ev = 1e300;
+    double bmin_ev = 1e300, bmin_prop = 1e300;
     for (int kw = 0; kw < (tr.k2 > 0.0 ? 2 : 1); ++kw) {
         // the second pass (derivative plans with k2) checks only for a Wood anomaly
         const double kc = kw == 0 ? k : tr.k2;
@@ -274,6 +276,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
                 if (b < bmin) bmin = b;
                 // the smallest evanescent b (attained at the smallest |alpha_n| > k, inside this box)
                 if (kw == 0 && aa > k && b < bmin_ev) bmin_ev = b;
+                if (kw == 0 && aa <= k && b < bmin_prop) bmin_prop = b;
             }
         if (bmin < 1e-8 * kc) return fail(GF_ERR_WOOD, "gf_plan: |beta_n| = %.3g < 1e-8 k (Wood anomaly)", bmin);
     }
@@ -312,6 +315,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     for (int i = 0; i < 3; ++i) p->M[i] = i < dim ? M[i] : 1;
     p->tr = tr;
     p->bmin_ev = bmin_ev;
+    p->bmin_prop = bmin_prop < 1e300 ? bmin_prop : 0.0;
     p->precision = tr.precision;
     p->kind = tr.kind;
     p->nf = tr.kind == GF_MAXWELL ? 7 : tr.kind == GF_DERIV2D ? (tr.k2 > 0.0 ? 6 : 3) : 1;
@@ -625,6 +629,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
             const bool want_exp = p->precision == GF_FP64;
             if ((e = gf_dev_alloc(&p->btab, ne * eb, st)) != cudaSuccess ||
                 (e = gf_dev_alloc((void **)&p->prop, sizeof(PropEntry) * nprop_max + 16, st)) != cudaSuccess ||
+                (e = gf_dev_alloc((void **)&p->trig, sizeof(longlong2) * GF_TRIG_STEPS, st)) != cudaSuccess ||
                 (want_exp && (e = gf_dev_alloc((void **)&p->exptab, 2 * sizeof(double2) * p->exptab_n, st)) != cudaSuccess)) {
                 st_err = fail(GF_ERR_NOMEM, "gf_plan: device allocation (series tables): %s", cudaGetErrorString(e));
                 break;
@@ -641,7 +646,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
             ea.btab = p->btab;
             ea.exptab_n = want_exp ? p->exptab_n : 0;
             ea.exptab_j0 = p->exptab_j0;
-            if ((e = gf_launch_series_tables(ea, p->precision, want_exp ? p->exptab : nullptr, p->prop, p->nprop_dev,
+            if ((e = gf_launch_series_tables(ea, p->precision, want_exp ? p->exptab : nullptr, p->trig, p->prop, p->nprop_dev,
                                              pbox, st)) != cudaSuccess) {
                 st_err = fail(GF_ERR_CUDA, "gf_plan: series table launch: %s", cudaGetErrorString(e));
                 break;
@@ -710,15 +715,16 @@ gf_status gf_eval_grid(gf_plan_t p, void *dev_out, size_t out_bytes, void *cuda_
 // target slots of the output's entries each).  With these the far sums are the
 // same bit for bit from call to call: the same list, and slab partials added in
 // slab order.
-constexpr int64_t GF_COUNTER_PAD = 1024;
+constexpr int64_t GF_COUNTER_PAD = 2304;
 static_assert(GF_SCRATCH_COUNTERS <= GF_COUNTER_PAD, "counter block too small");
 
 // Segments of the stable far list: 512 targets, more when that would make over
-// 8192 segments (the scan's work per bucket stays bounded).
+// 1024 segments (the scan's work per bucket and the segments' counts, 4 KiB each,
+// stay bounded).
 static int64_t far_segment_size(int64_t n)
 {
     const int64_t segs = (n + 511) / 512;
-    return segs <= 8192 ? 512 : ((n + 8191) / 8192 + 31) / 32 * 32;
+    return segs <= 1024 ? 512 : ((n + 1023) / 1024 + 31) / 32 * 32;
 }
 
 gf_status gf_eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int which, void *dev_out,
@@ -732,13 +738,25 @@ gf_status gf_eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int whic
     // to the pool in stream order after the kernels: concurrent calls on other
     // streams each have their own, and the plan stays unchanged
     const bool slabs = p->dim == 3;
-    const int64_t npad = (n + 31) / 32 * 32, nchmax = npad / 32, slabcap = 2 * npad;
+    // slab partials: two slots per target, up to 32 for short lists (they use more slabs)
+    const int64_t npad = (n + 31) / 32 * 32, nchmax = npad / 32, slabcap = npad <= (1 << 14) ? 32 * npad : std::max<int64_t>(2 * npad, 1 << 19);
     const int64_t segsize = far_segment_size(n), nseg = (n + segsize - 1) / segsize;
     const size_t ints = (size_t)(GF_COUNTER_PAD + 3 * n + (slabs ? 2 * nchmax + nseg * GF_FAR_BUCKETS : 0));
     const size_t off_buf = (sizeof(int) * ints + 255) / 256 * 256;
     const size_t buf_bytes = slabs ? (size_t)slabcap * gf_out_entries(which) * p->elem : 0;
+    // far targets by matrix products: from gf_far_product_min targets on, propagating indices
+    // within the one block of rows that the products give them (k < 7), no far-region grid
+    size_t mma_bytes = 0;
+    int mma_cells = 0;
+    if (slabs && n >= gf_far_product_min(p->precision, p->nf) && p->k < 7.0 && !p->fargrid && which != GF_OUT_LD)
+        mma_bytes = gf_far_product_bytes(p->precision, n, p->nf == 1 ? 1 : gf_out_entries(which), &mma_cells);
+    const size_t off_mma = (off_buf + 2 * buf_bytes + 255) / 256 * 256;
     int *scratch = nullptr;
-    CU(gf_dev_alloc((void **)&scratch, off_buf + 2 * buf_bytes, st));
+    CU(gf_dev_alloc((void **)&scratch, off_mma + mma_bytes, st));
+    if (mma_bytes) {
+        a.mma = (char *)scratch + off_mma;
+        a.mma_cells = mma_cells;
+    }
     a.far_count = scratch;
     a.far_idx = scratch + GF_COUNTER_PAD;
     a.far_sorted = a.far_idx + n;
@@ -831,6 +849,9 @@ gf_status gf_plan_eval_args(gf_plan_t p, const double *dev_xyz, int64_t n, int w
     a.exptab_n = p->exptab_n;
     a.exptab_j0 = p->exptab_j0;
     a.bmin = p->bmin_ev;
+    a.bprop = p->bmin_prop;
+    a.err = p->errw;
+    a.trig = p->trig;
     a.nyqgrid = p->nyqgrid;
     a.fargrid = p->fargrid;
     if (p->fargrid) {
@@ -984,7 +1005,7 @@ gf_status gf_destroy(gf_plan_t p)
     // the plan may have been used on any stream: wait for the device, then hand
     // the buffers back to the pool
     cudaDeviceSynchronize();
-    void *bufs[] = {p->grid, p->nyqgrid, p->fargrid, p->tables, p->btab, p->prop, p->exptab, p->errw};
+    void *bufs[] = {p->grid, p->nyqgrid, p->fargrid, p->tables, p->btab, p->prop, p->exptab, p->trig, p->errw};
     for (void *b : bufs) gf_dev_free(b, 0);
     for (int i = 0; i < 6; ++i)
         if (p->ev[i]) cudaEventDestroy(p->ev[i]);
