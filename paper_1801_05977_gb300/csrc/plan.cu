@@ -441,7 +441,8 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     const size_t nodes_padded = (size_t)p->P1 * p->P2 * p->P3;
     p->grid_bytes = nodes_padded * p->nf * p->elem;
     const size_t E_n = (size_t)Mlast * Q;
-    const size_t host_tab_bytes = sizeof(double) * 5 * Q + sizeof(double2) * Q + (deriv ? sizeof(double) * 4 * Q : 0);
+    const int Qa = 5 * Q + (Q & 1);  // the five real tables, rounded up so that the complex ones lie on 16 bytes
+    const size_t host_tab_bytes = sizeof(double) * Qa + sizeof(double2) * Q + (deriv ? sizeof(double) * 4 * Q : 0);
     const bool ftabs = tr.precision == GF_FP32_SPLIT;  // float copies for the split plans' coefficients
     const size_t dcheb_n = deriv ? 3 * hcheb_n : 0;
     const size_t tab_bytes = host_tab_bytes + sizeof(double2) * (E_n + hcheb_n + dcheb_n) +
@@ -464,12 +465,12 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
         }
         char *tb = (char *)p->tables;
         double *d_tt = (double *)tb, *d_tW = d_tt + Q, *d_rr = d_tW + Q, *d_P0 = d_rr + Q, *d_P1 = d_P0 + Q;
-        double2 *d_B = (double2 *)(d_P1 + Q);
+        double2 *d_B = (double2 *)(d_tt + Qa);
         double *d_rrd = (double *)(d_B + Q), *d_wyd = d_rrd + (deriv ? 2 * Q : 0);
         double2 *d_E = (double2 *)(d_wyd + (deriv ? 2 * Q : 0)), *d_H = d_E + E_n, *d_D = d_H + hcheb_n;
         float2 *d_Ef = ftabs ? (float2 *)(d_D + dcheb_n) : nullptr, *d_Hf = ftabs ? d_Ef + E_n : nullptr;
         {
-            std::vector<char> pack(host_tab_bytes);
+            std::vector<char> pack(host_tab_bytes, 0);
             char *hb = pack.data();
             memcpy(hb + ((char *)d_tt - tb), tt.data(), sizeof(double) * Q);
             memcpy(hb + ((char *)d_tW - tb), tW.data(), sizeof(double) * Q);
