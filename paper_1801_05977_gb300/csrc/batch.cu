@@ -87,7 +87,7 @@ static gf_status batch_synth_setup(gf_batch_t b)
         gf_synth_config(a, b->precision, b->tune.tj_max, sm);
         for (int i = 0; i < 3; ++i) smax[i] = sm[i] > smax[i] ? sm[i] : smax[i];
         const int ncols = a.M1 * a.M2;
-        b->h_prefix[0][p + 1] = b->h_prefix[0][p] + ncols / a.TJ;
+        b->h_prefix[0][p + 1] = b->h_prefix[0][p] + a.ndbl + ncols / a.TJ;
         b->h_prefix[1][p + 1] = b->h_prefix[1][p] + (a.M1 / a.TJ2) * (a.L3count + a.nyq) * a.nf;
         b->h_prefix[2][p + 1] = b->h_prefix[2][p] + (a.L3count + a.nyq) * a.M2 / a.RB1;
     }
@@ -102,6 +102,7 @@ static gf_status batch_synth_setup(gf_batch_t b)
         b->sb.smem[i] = smax[i];
         int tot = b->h_prefix[i][b->np];
         int g = b->nsm * 4;
+        if (i == 0) b->sb.total0 = tot;
         b->sb.grid[i] = tot < g ? tot : g;
     }
     return GF_OK;

@@ -102,11 +102,11 @@ struct SynthArgs {
     const double *tW;   // [Q] w_m hw X'(t_m) on [c, (c+c~)/2]
     const double *tt;   // [Q] t_m
     const double2 *E;   // [Mlast][Q] e^{i q_b t_m}, q_b = freq(b) pi / c~
-    const float2 *Ef;   // the same in float (split plans)
+    const float2 *Ef;   // the same in float, [Q][GF_EF_ROW(Mlast)], b <= Mlast/2 (3D split plans)
     const double *rr;   // [Q] r_m on [eps, 2 eps]
     const double2 *B;   // [Q] 3D: w_m hw e^{i k r_m}(2 i k Y'(r_m) + Y''(r_m))
-    const double2 *hcheb; // Chebyshev coefficients per panel [hnpan][hdeg + 1]: 3D h(s); 2D (S0, S1)(eta)
-    const float2 *hchebf; // the same in float (split plans)
+    const double2 *hcheb; // Chebyshev interpolants per panel, by powers of x, [hnpan][hdeg + 1]: 3D h(s); 2D (S0, S1)(eta)
+    const float2 *hchebf; // the same in float, [hdeg + 1][hnpan] (3D split plans)
     int hdeg, hnpan;
     double hpan, ihpan; // panel width in s and its inverse
     const double *Pw0;  // [Q] 2D: w_m hw Phi_1(r_m) r_m      (J0 weights)
@@ -141,6 +141,9 @@ struct SynthArgs {
     int deriv;
     double k2;
     const double2 *dcheb;
+    // 3D split plans: the columns formed in double lie in the box n1 = dbx0 ..
+    // dbx0 + dbw - 1, n2 from dby0, ndbl columns in all (0 in other plans)
+    int dbx0, dbw, dby0, ndbl;
 };
 
 // Complex entries per target of an output selection (gf_eval_points `which`).
@@ -278,6 +281,7 @@ struct SynthBatch {
     const int *prefix[3];
     int np;
     int grid[3];
+    int total0;             // virtual blocks of the first pass
     size_t smem[3];
 };
 struct EvalBatch {
@@ -289,6 +293,27 @@ struct EvalBatch {
     int scatter_per_pair;
     bool near_lists;        // per-pair near lists present (EvalArgs::near_idx): classify, then near3d_list_batch
 };
+
+// degree of the panels' interpolants; row length of SynthArgs::Ef
+constexpr int GF_HDEG = 14;
+__host__ __device__ constexpr int GF_EF_ROW(int n) { return ((n >> 1) + 8) & ~7; }
+
+// One panel's polynomial (two real functions packed in a double2) at x in [-1, 1].
+__device__ __forceinline__ double2 poly_eval(const double2 *c, int deg, double x)
+{
+    double2 v = c[deg];
+    for (int k = deg - 1; k >= 0; --k) {
+        const double2 ck = c[k];
+        v.x = fma(v.x, x, ck.x);
+        v.y = fma(v.y, x, ck.y);
+    }
+    return v;
+}
+
+// synthsplit.cu: first pass of the 3D split plans (sets a.TJ; returns the CTAs' shared memory)
+size_t gf_first_split_config(SynthArgs &a, int tj_max);
+cudaError_t gf_launch_first_split(const SynthArgs &a, size_t smem, cudaStream_t s);
+cudaError_t gf_launch_first_split_batch(const SynthBatch &b, int nsm, cudaStream_t s);
 
 // launch helpers implemented in synth.cu / eval.cu
 cudaError_t gf_launch_synth(const SynthArgs &a, int precision, cudaStream_t s);

@@ -406,7 +406,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     // radial transforms on [0, s_max], s_max >= the largest frequency norm:
     // 3D h(s) = sum_m B_m sin(s r_m)/s, 2D the Bessel sums of F1-hat, F2-hat.
     // (computed on the device from the quadrature tables, see gf_launch_cheb_table)
-    const int hdeg = 14;
+    const int hdeg = GF_HDEG;
     const double hpan = 2.0;
     int hnpan = 1;
     size_t hcheb_n = 0;
@@ -443,7 +443,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     const size_t E_n = (size_t)Mlast * Q;
     const int Qa = 5 * Q + (Q & 1);  // the five real tables, rounded up so that the complex ones lie on 16 bytes
     const size_t host_tab_bytes = sizeof(double) * Qa + sizeof(double2) * Q + (deriv ? sizeof(double) * 4 * Q : 0);
-    const bool ftabs = tr.precision == GF_FP32_SPLIT;  // float copies for the split plans' coefficients
+    const bool ftabs = dim == 3 && tr.precision == GF_FP32_SPLIT;  // float copies for the split plans' coefficients
     const size_t dcheb_n = deriv ? 3 * hcheb_n : 0;
     const size_t tab_bytes = host_tab_bytes + sizeof(double2) * (E_n + hcheb_n + dcheb_n) +
                              (ftabs ? sizeof(float2) * (E_n + hcheb_n) : 0);
@@ -547,6 +547,16 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
         sa.deriv = deriv ? 1 : 0;
         sa.k2 = tr.k2;
         sa.dcheb = deriv ? d_D : nullptr;
+        if (ftabs) {
+            // the box around |alpha_n| < sqrt(k^2 + gfloat^2), clipped to the grid's indices
+            const double R = sqrt(k * k + sa.gfloat * sa.gfloat) * (1.0 + 1e-12);
+            auto lo = [&](double al, int M) { return std::max((int)fmax(floor(-al - R), -1e6), -M / 2); };
+            auto hi = [&](double al, int M) { return std::min((int)fmin(ceil(-al + R), 1e6), M / 2 - 1); };
+            sa.dbx0 = lo(a1, sa.M1);
+            sa.dby0 = lo(a2, sa.M2);
+            sa.dbw = std::max(hi(a1, sa.M1) - sa.dbx0 + 1, 0);
+            sa.ndbl = sa.dbw * std::max(hi(a2, sa.M2) - sa.dby0 + 1, 0);
+        }
         {
             // one CTA holds whole lines of every stored field in shared memory
             int dev = 0, optin = 232448;

@@ -72,23 +72,6 @@ __device__ __forceinline__ double2 xprime_terms(double2 beta, double q, const do
     return T12;
 }
 
-// Clenshaw sum of one panel's Chebyshev coefficients (two real functions packed
-// in a double2) at x in [-1, 1].
-__device__ __forceinline__ double2 cheb_eval(const double2 *cc, int deg, double x)
-{
-    double b1r = 0.0, b1i = 0.0, b2r = 0.0, b2i = 0.0;
-    for (int kk = deg; kk >= 1; --kk) {
-        const double2 ck = cc[kk];
-        const double tr = fma(2.0 * x, b1r, ck.x - b2r);
-        const double ti = fma(2.0 * x, b1i, ck.y - b2i);
-        b2r = b1r;
-        b2i = b1i;
-        b1r = tr;
-        b1i = ti;
-    }
-    return make_double2(fma(x, b1r, cc[0].x - b2r), fma(x, b1i, cc[0].y - b2i));
-}
-
 // e^{2 pi i m/n} for 0 <= m < n from the table of the first half (tw[m] =
 // e^{2 pi i m/n}, m < n/2): the second half is its negative.
 template <typename C>
@@ -270,9 +253,9 @@ __device__ void deriv_fields_2d(const SynthArgs &a, C *buf0, int TJ, int t, int 
     const double ip = 2.0 * GF_PI, al = a.a1, kk = a.k * a.k, c1 = al + jx;
     const int nd = a.hdeg + 1;
     const size_t tab = (size_t)a.hnpan * nd;
-    const double2 d0 = cheb_eval(a.dcheb + (size_t)pnl * nd, a.hdeg, x);            // (Q1, R0)
-    const double2 d1 = cheb_eval(a.dcheb + tab + (size_t)pnl * nd, a.hdeg, x);      // (R2, S1)
-    const double S3 = cheb_eval(a.dcheb + 2 * tab + (size_t)pnl * nd, a.hdeg, x).x;  // S3
+    const double2 d0 = poly_eval(a.dcheb + (size_t)pnl * nd, a.hdeg, x);            // (Q1, R0)
+    const double2 d1 = poly_eval(a.dcheb + tab + (size_t)pnl * nd, a.hdeg, x);      // (R2, S1)
+    const double S3 = poly_eval(a.dcheb + 2 * tab + (size_t)pnl * nd, a.hdeg, x).x;  // S3
     double cp = 0.0, sp = 0.0, f2i = 0.0, f2yi = 0.0;
     if (eta > 0.0) {
         cp = jx / eta;
@@ -322,23 +305,9 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
     C *buf0 = tw + (n >> 1);                             // [nf][TJ][n]
     C *buf1 = buf0 + nf * TJ * n;                      // [TJ][n] scratch of the transforms
     double *A2s = reinterpret_cast<double *>(buf1 + TJ * n); // [TJ]
-    // split plans, float coefficients: A_m [TJ][Q] (16-byte aligned so that the X'-integral
-    // loop reads it four nodes at a time), |alpha_j|^2 in float [TJ]
-    float *Avf = reinterpret_cast<float *>(reinterpret_cast<uintptr_t>(A2s + TJ + 1) & ~(uintptr_t)15);
-    float *A2f = Avf + ((TJ * Q + 3) & ~3);
-    // float-column data: |alpha_j|^2 - k^2 and q_b^2 as float pairs (hi, lo), g in
-    // float, and per column bit 0 = X'-integrals skipped, bit 1 = float coefficient
-    float2 *A2mkf = reinterpret_cast<float2 *>((reinterpret_cast<uintptr_t>(A2f + TJ) + 15) & ~(uintptr_t)15);
-    float2 *qqf = A2mkf + TJ;
-    float *gcol = reinterpret_cast<float *>(qqf + n);
-    int *cflag = reinterpret_cast<int *>(gcol + TJ);
-    // float copies of the quadrature weights and nodes [Q] each, q_b in float [n]
-    float *tWs = reinterpret_cast<float *>(cflag + TJ);
-    float *tts = tWs + Q;
-    float *qfs = tts + Q;
     // 2D derivative plans with a second wave number: its A_m [TJ][Q] and beta [TJ]
     const bool need_k2 = DERIV && a.k2 > 0.0;
-    double2 *Av2 = reinterpret_cast<double2 *>((reinterpret_cast<uintptr_t>(qfs + n) + 15) & ~(uintptr_t)15);
+    double2 *Av2 = reinterpret_cast<double2 *>((reinterpret_cast<uintptr_t>(A2s + TJ) + 15) & ~(uintptr_t)15);
     double2 *betas2 = Av2 + TJ * Q;
     const int ncols = (a.dim == 3) ? a.M1 * a.M2 : a.M1;
     // tiles alternately from both ends of the column range: the low frequencies
@@ -346,7 +315,6 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
     // they are scheduled first and the last wave holds the cheap middle
     const int ntiles = ncols / TJ;
     const int col0 = ((blk & 1) ? ntiles - 1 - (blk >> 1) : (blk >> 1)) * TJ;
-    const bool fcoef = sizeof(R) == 4 && a.dim == 3;
 
     load_twiddles<R>(tw, n);
     for (int t = threadIdx.x; t < TJ; t += blockDim.x) {
@@ -365,46 +333,10 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
         const double2 bt = beta_of(a.k, A2);
         betas[t] = bt;
         if (need_k2) betas2[t] = beta_of(a.k2, A2);
-        if (fcoef) {
-            const double d = A2 - a.k * a.k;
-            A2f[t] = (float)A2;
-            const float h = (float)d;
-            A2mkf[t] = make_float2(h, (float)(d - (double)h));
-            gcol[t] = (float)bt.y;
-            cflag[t] = (bt.y > a.gskip ? 1 : 0) | (bt.y >= a.gfloat ? 2 : 0);
-        }
-    }
-    if (fcoef) {
-        // q_b = j q_s and q_b^2 as float pairs from q_s's pair (qsh, qsl), with no
-        // double operation: j q_sh by TwoProd (j is an integer below 2^12), then the
-        // square of the pair (its l^2 term dropped), about 2^-46 relative
-        for (int b = threadIdx.x; b < n; b += blockDim.x) {
-            const float jf = (float)freq_of(b, n);
-            const float ph = jf * a.qsh;
-            const float pl = __fmaf_rn(jf, a.qsh, -ph) + jf * a.qsl;
-            const float h = ph * ph;
-            const float l = __fmaf_rn(ph, ph, -h) + 2.0f * ph * pl;
-            const float s = h + l;
-            qqf[b] = make_float2(s, l - (s - h));
-            qfs[b] = ph + pl;
-        }
-        for (int m = threadIdx.x; m < Q; m += blockDim.x) {
-            tWs[m] = (float)a.tW[m];
-            tts[m] = (float)a.tt[m];
-        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < TJ * Q; i += blockDim.x) {
         int t = i / Q, m = i - t * Q;
-        if (fcoef) {
-            // the column's flags: bit 0 skipped X'-integrals, bit 1 float coefficient
-            const int f = cflag[t];
-            if (f & 1) continue;
-            if (f & 2) {
-                Avf[i] = tWs[m] * expf(-gcol[t] * tts[m]);
-                continue;
-            }
-        }
         double2 b = betas[t];
         if (b.y > a.gskip) continue;  // this column's X'-integrals are not used
         double tm = a.tt[m];
@@ -437,8 +369,6 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
     __syncthreads();
 
     const double k2 = a.k * a.k, ik2 = 1.0 / k2;
-    // the float branch's constants, converted once
-    const float ihpanf = (float)a.ihpan, hpanf = (float)a.hpan, invVf = (float)a.invV;
     // The coefficients are even in the last-axis index j (they depend on q_j
     // through q_j^2, and the two X' terms of Eqs. (fck-coef)/(kdj1) trade places
     // under q -> -q), except the Maxwell xz and yz fields, whose factor c^3 = q_j
@@ -447,89 +377,11 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
     // below from b' = n - b (j' = -j).
     // items: (t, b) for b < n/2 by shift and mask, then the Nyquist b = n/2 of each column
     const int nh = (n >> 1) + 1, lgh = lg - 1, nlow = TJ << lgh;
-    const float hmaxf = (float)(a.hnpan - 1);
     for (int i = threadIdx.x; i < TJ * nh; i += blockDim.x) {
         const bool low = i < nlow;
         const int t = low ? (i >> lgh) : i - nlow, b = low ? (i & ((n >> 1) - 1)) : (n >> 1);
         int col = col0 + t;
         int jl = freq_of(b, n);
-        if (fcoef && (cflag[t] & 2)) {
-            // Split plans, evanescent column clear of Wood anomalies (g >= gfloat):
-            // the coefficient in float, with no double operation.  D = |xi|^2 - k^2
-            // (small near the resonance sphere) is the sum of two float pairs, exact
-            // to ~2^-46 relative to its terms (Knuth's TwoSum), then rounded: since
-            // |D| >= 1e-6 k^2 (the resonance rule), this is below float rounding of D.
-            // Every other factor is O(1) in relative terms.
-            const float qf = qfs[b];
-            const float g = gcol[t];
-            float T12f = 0.f;
-            if (!(cflag[t] & 1)) {
-                const float *Am = Avf + t * Q;
-                const float2 *Em = a.Ef + (size_t)b * Q;
-                float s1 = 0.f, s3 = 0.f;
-                int m = 0;
-                if ((Q & 3) == 0) {
-                    // four nodes per step: one 16-byte shared load of A, two of E
-                    const float4 *A4 = reinterpret_cast<const float4 *>(Am);
-                    const float4 *E4 = reinterpret_cast<const float4 *>(Em);
-                    for (int m4 = 0; m4 < (Q >> 2); ++m4) {
-                        const float4 A = A4[m4], E01 = __ldg(E4 + 2 * m4), E23 = __ldg(E4 + 2 * m4 + 1);
-                        s1 = fmaf(A.x, E01.x, s1);
-                        s3 = fmaf(A.x, E01.y, s3);
-                        s1 = fmaf(A.y, E01.z, s1);
-                        s3 = fmaf(A.y, E01.w, s3);
-                        s1 = fmaf(A.z, E23.x, s1);
-                        s3 = fmaf(A.z, E23.y, s3);
-                        s1 = fmaf(A.w, E23.z, s1);
-                        s3 = fmaf(A.w, E23.w, s3);
-                    }
-                    m = Q;
-                }
-                for (; m < Q; ++m) {
-                    const float A = Am[m];
-                    const float2 E = Em[m];
-                    s1 = fmaf(A, E.x, s1);
-                    s3 = fmaf(A, E.y, s3);
-                }
-                T12f = (g * s1 - qf * s3) * __frcp_rn(g * (g * g + qf * qf));
-            }
-            const float2 Ad = A2mkf[t], Qd = qqf[b];
-            const float dh = __fadd_rn(Ad.x, Qd.x), dv = __fsub_rn(dh, Ad.x);
-            const float de = __fadd_rn(__fsub_rn(Ad.x, __fsub_rn(dh, dv)), __fsub_rn(Qd.x, dv));
-            const float iD = __frcp_rn(__fadd_rn(dh, __fadd_rn(de, __fadd_rn(Ad.y, Qd.y))));
-            // |xi| by the hardware reciprocal square root (its ~2^-23 relative error moves
-            // the Chebyshev point by less than the float rounding of h)
-            const float s2 = fmaf(qf, qf, A2f[t]);
-            const float sf = s2 > 0.f ? s2 * rsqrtf(s2) : 0.f;
-            const float pf = fminf(floorf(sf * ihpanf), hmaxf);
-            const int pnl = (int)pf;
-            const float x = (sf - (pf + 0.5f) * hpanf) * (2.0f / hpanf);
-            const float2 *cc = a.hchebf + (size_t)pnl * (a.hdeg + 1);
-            float b1r = 0.f, b1i = 0.f, b2r = 0.f, b2i = 0.f;
-            for (int kk = a.hdeg; kk >= 1; --kk) {
-                const float2 ck = cc[kk];
-                const float tr = fmaf(2.0f * x, b1r, ck.x - b2r);
-                const float ti = fmaf(2.0f * x, b1i, ck.y - b2i);
-                b2r = b1r;
-                b2i = b1i;
-                b1r = tr;
-                b1i = ti;
-            }
-            const float hr = fmaf(x, b1r, cc[0].x - b2r), hi = fmaf(x, b1i, cc[0].y - b2i);
-            const float cr = fmaf(hr, iD, T12f) * invVf, ci = hi * iD * invVf;
-            if (nf == 1) {
-                buf0[t * n + b] = cmk((R)cr, (R)ci);
-            } else {
-                const int jx = freq_of(col % a.M1, a.M1), jy = freq_of(col / a.M1, a.M2);
-                const float ik2f = (float)ik2;
-                const float cv0 = (float)(a.a1 + jx), cv1 = (float)(a.a2 + jy), cv2 = qf;
-                const float f[7] = {1.f - cv0 * cv0 * ik2f, 1.f - cv1 * cv1 * ik2f, 1.f - cv2 * cv2 * ik2f,
-                                    -cv0 * cv1 * ik2f,      -cv0 * cv2 * ik2f,      -cv1 * cv2 * ik2f, 1.f};
-#pragma unroll
-                for (int e = 0; e < 7; ++e) buf0[(e * TJ + t) * n + b] = cmk((R)(f[e] * cr), (R)(f[e] * ci));
-            }
-            continue;
-        }
         const double2 beta = betas[t];
         double q = (double)jl * a.qs;
         double A2 = A2s[t];
@@ -545,21 +397,9 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
             double s = sqrt(A2 + q * q);
             int pnl = min((int)(s * a.ihpan), a.hnpan - 1);
             double x = (s - (pnl + 0.5) * a.hpan) * (2.0 / a.hpan);
-            const double2 *cc = a.hcheb + (size_t)pnl * (a.hdeg + 1);
-            double b1r = 0.0, b1i = 0.0, b2r = 0.0, b2i = 0.0;
-            for (int kk = a.hdeg; kk >= 1; --kk) {
-                double2 ck = cc[kk];
-                double tr = fma(2.0 * x, b1r, ck.x - b2r);
-                double ti = fma(2.0 * x, b1i, ck.y - b2i);
-                b2r = b1r;
-                b2i = b1i;
-                b1r = tr;
-                b1i = ti;
-            }
-            double hr = fma(x, b1r, cc[0].x - b2r);
-            double hi = fma(x, b1i, cc[0].y - b2i);
+            const double2 h = poly_eval(a.hcheb + (size_t)pnl * (a.hdeg + 1), a.hdeg, x);
             const double iD = 1.0 / D;
-            Cj = make_double2(fma(hr, iD, T12.x), fma(hi, iD, T12.y));
+            Cj = make_double2(fma(h.x, iD, T12.x), fma(h.y, iD, T12.y));
         } else {
             int jx = freq_of(col, a.M1);
             double2 K = make_double2(1.0 / D + T12.x, T12.y);
@@ -574,19 +414,8 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
                 double eta = sqrt(eta2);
                 int pnl = min((int)(eta * a.ihpan), a.hnpan - 1);
                 double x = (eta - (pnl + 0.5) * a.hpan) * (2.0 / a.hpan);
-                const double2 *cc = a.hcheb + (size_t)pnl * (a.hdeg + 1);
-                double b1r = 0.0, b1i = 0.0, b2r = 0.0, b2i = 0.0;
-                for (int kk = a.hdeg; kk >= 1; --kk) {
-                    double2 ck = cc[kk];
-                    double tr = fma(2.0 * x, b1r, ck.x - b2r);
-                    double ti = fma(2.0 * x, b1i, ck.y - b2i);
-                    b2r = b1r;
-                    b2i = b1i;
-                    b1r = tr;
-                    b1i = ti;
-                }
-                const double S0 = fma(x, b1r, cc[0].x - b2r);
-                const double S1 = fma(x, b1i, cc[0].y - b2i);
+                const double2 S = poly_eval(a.hcheb + (size_t)pnl * (a.hdeg + 1), a.hdeg, x);
+                const double S0 = S.x, S1 = S.y;
                 // F1 = (1 + Phi1-hat/(2 pi))/eta^2,  Phi1-hat/(2 pi) = S0
                 F1 = make_double2((1.0 + S0) / eta2, 0.0);
                 // F2 = (-2 i j1 F1 + Phi2-hat/(2 pi))/eta^2,  Phi2-hat/(2 pi) = -i (j1/eta) S1
@@ -999,22 +828,18 @@ void synth_config_t(SynthArgs &a, int tj_max, size_t sm[3])
 {
     typedef typename cplx_t<R>::T C;
     const int ncols = (a.dim == 3) ? a.M1 * a.M2 : a.M1;
-    // per column: A_m (double2 and float), beta, |alpha|^2 (double), |alpha|^2 - k^2, its float;
-    // float-column data (|alpha|^2 - k^2 as a float pair, g, flags); per b: twiddles, q_b^2
-    // and its float pair, q_b in float; the quadrature weights and nodes in float; plus the
-    // two line buffers
+    // per column: A_m, beta, |alpha|^2 and the line buffers (every field's, one of scratch); the twiddles
     auto bytes = [&](int TJ) {
-        return sizeof(C) * (a.Mlast / 2) + sizeof(double) * a.Mlast + sizeof(float2) * a.Mlast +
-               TJ * (sizeof(double2) * a.Q + sizeof(double2) + 2 * sizeof(double) + sizeof(float)) +
-               TJ * (sizeof(float2) + sizeof(float) + sizeof(int)) +
-               sizeof(float) * ((TJ * a.Q + 3) & ~3) + sizeof(C) * (a.nf + 1) * TJ * a.Mlast + 64 +
-               sizeof(float) * (2 * a.Q + a.Mlast) + 16 +
+        return sizeof(C) * (a.Mlast / 2) + TJ * (sizeof(double2) * a.Q + sizeof(double2) + sizeof(double)) +
+               sizeof(C) * (a.nf + 1) * TJ * a.Mlast + 16 +
                (a.deriv && a.k2 > 0.0 ? TJ * sizeof(double2) * (a.Q + 1) + 16 : 0);
     };
     int TJ = tj_max;
     while (TJ > 1 && (TJ > ncols || bytes(TJ) > 160 * 1024)) TJ >>= 1;
     a.TJ = TJ;
     sm[0] = bytes(TJ);
+    // 3D split plans have a first pass of their own (wider tiles: its columns are the lanes)
+    if (sizeof(R) == 4 && a.dim == 3) sm[0] = gf_first_split_config(a, 4 * tj_max);
     int TJ2 = 8;
     while (TJ2 > 1 && (TJ2 > a.M1 || sizeof(C) * (a.M2 / 2 + 2 * TJ2 * a.M2) > 160 * 1024)) TJ2 >>= 1;
     a.TJ2 = TJ2;
@@ -1090,7 +915,9 @@ cudaError_t launch_synth_t(const SynthArgs &a0, cudaStream_t s)
     synth_config_t<R>(a, sizeof(R) == 4 ? 16 : 8, sm);
     const int ncols = (a.dim == 3) ? a.M1 * a.M2 : a.M1;
     cudaError_t e;
-    if (a.deriv) {
+    if (sizeof(R) == 4 && a.dim == 3) {
+        if ((e = gf_launch_first_split(a, sm[0], s)) != cudaSuccess) return e;
+    } else if (a.deriv) {
         e = cudaFuncSetAttribute(synth_first_pass<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm[0]);
         if (e != cudaSuccess) return e;
         synth_first_pass<R, true><<<ncols / a.TJ, 256, sm[0], s>>>(a);
@@ -1099,7 +926,7 @@ cudaError_t launch_synth_t(const SynthArgs &a0, cudaStream_t s)
         if (e != cudaSuccess) return e;
         synth_first_pass<R, false><<<ncols / a.TJ, 256, sm[0], s>>>(a);
     }
-    gf_count_launch(1);
+    if (!(sizeof(R) == 4 && a.dim == 3)) gf_count_launch(1);
     if (a.dim == 3) {
         e = launch_x2<R>(a, sm[1], s);
         if (e != cudaSuccess) return e;
@@ -1116,8 +943,9 @@ template <typename R>
 cudaError_t launch_synth_batch_t(const SynthBatch &b, cudaStream_t s)
 {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(synth_first_pass_batch<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)b.smem[0])) != cudaSuccess ||
+    if ((sizeof(R) == 8 &&
+         (e = cudaFuncSetAttribute(synth_first_pass_batch<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)b.smem[0])) != cudaSuccess) ||
         (e = cudaFuncSetAttribute(synth_x2_pass_batch<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)b.smem[1])) != cudaSuccess ||
         (e = cudaFuncSetAttribute(synth_x1_pass_batch<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1136,13 +964,18 @@ cudaError_t launch_synth_batch_t(const SynthBatch &b, cudaStream_t s)
         return want < per * nsm ? want : per * nsm;
     };
     int per[3] = {0, 0, 0};
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[0], synth_first_pass_batch<R>, 256, b.smem[0]);
+    if (sizeof(R) == 8) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[0], synth_first_pass_batch<double>, 256, b.smem[0]);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[1], synth_x2_pass_batch<R>, 256, b.smem[1]);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per[2], synth_x1_pass_batch<R>, 256, b.smem[2]);
-    synth_first_pass_batch<R><<<resident(per[0], b.grid[0]), 256, b.smem[0], s>>>(b.args, b.prefix[0], b.np);
+    if (sizeof(R) == 8) {
+        synth_first_pass_batch<double><<<resident(per[0], b.grid[0]), 256, b.smem[0], s>>>(b.args, b.prefix[0], b.np);
+        gf_count_launch(1);
+    } else if ((e = gf_launch_first_split_batch(b, nsm, s)) != cudaSuccess) {
+        return e;
+    }
     synth_x2_pass_batch<R><<<resident(per[1], b.grid[1]), 256, b.smem[1], s>>>(b.args, b.prefix[1], b.np);
     synth_x1_pass_batch<R><<<resident(per[2], b.grid[2]), 256, b.smem[2], s>>>(b.args, b.prefix[2], b.np);
-    gf_count_launch(3);
+    gf_count_launch(2);
     return cudaGetLastError();
 }
 
@@ -1154,10 +987,36 @@ cudaError_t gf_launch_synth(const SynthArgs &a, int precision, cudaStream_t s)
 }
 
 namespace {
+// Integer coefficients of the Chebyshev polynomials: T_k(x) = sum_t c[k][t] x^t.
+struct ChebPowers {
+    double c[GF_HDEG + 1][GF_HDEG + 1];
+};
+constexpr ChebPowers cheb_powers()
+{
+    ChebPowers m{};
+    m.c[0][0] = 1.0;
+    m.c[1][1] = 1.0;
+    for (int k = 2; k <= GF_HDEG; ++k)
+        for (int t = 0; t <= k; ++t) m.c[k][t] = (t ? 2.0 * m.c[k - 1][t - 1] : 0.0) - m.c[k - 2][t];
+    return m;
+}
+__constant__ ChebPowers c_cheb_powers = cheb_powers();
+
+// Coefficient of x^t of the Chebyshev sum with coefficients c[k stride].  The
+// tables are stored by powers of x: Horner takes half of Clenshaw's operations.
+// The functions have bandwidth 2 eps < pi in s on panels of half-width 1, so the
+// Chebyshev coefficients fall like (eps/2)^k/k! and the sums over k do not cancel.
+__device__ __forceinline__ double to_power(const double *c, int stride, int t)
+{
+    double s = 0.0;
+    for (int k = GF_HDEG; k >= t; --k) s = fma(c_cheb_powers.c[k][t], c[k * stride], s);
+    return s;
+}
+
 // Piecewise Chebyshev interpolants of the radial transforms, one CTA per panel
 // [p w, (p+1) w]: values at the nn <= 16 Chebyshev points (sixteen threads per
 // point share the quadrature sum, reduced by shuffles), then the discrete
-// cosine transform to coefficients.
+// cosine transform to coefficients, stored by powers of the panel's x.
 //   3D: h(s) = sum_m B_m sin(s r_m)/s (complex).
 //   2D: (S0, S1)(s) = (sum_m P0_m J0(s r_m), sum_m P1_m J1(s r_m)) (two real functions).
 template <int DIM>
@@ -1166,6 +1025,7 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(const double *rr, const
                                                          float2 *outf)
 {
     __shared__ double2 fv[16];
+    __shared__ double cv[16][2];
     const int p = blockIdx.x, t = threadIdx.x, k = t >> 4, g = t & 15;
     const double cen = (p + 0.5) * w, hh = 0.5 * w;
     double ar = 0.0, ai = 0.0, s = 0.0;
@@ -1203,8 +1063,14 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(const double *rr, const
             ci = fma(fv[q].y, c, ci);
         }
         const double sc = (t == 0 ? 1.0 : 2.0) / nn;
-        out[(size_t)p * nn + t] = make_double2(cr * sc, ci * sc);
-        if (outf) outf[(size_t)p * nn + t] = make_float2((float)(cr * sc), (float)(ci * sc));
+        cv[t][0] = cr * sc;
+        cv[t][1] = ci * sc;
+    }
+    __syncthreads();
+    if (t < nn) {
+        const double2 c = make_double2(to_power(&cv[0][0], 2, t), to_power(&cv[0][1], 2, t));
+        out[(size_t)p * nn + t] = c;
+        if (outf) outf[(size_t)t * gridDim.x + p] = make_float2((float)c.x, (float)c.y);
     }
 }
 // The 2D derivative plans' Hankel transforms of the cutoff Y on the same panels:
@@ -1217,7 +1083,7 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(const double *rr, const
 __global__ void __launch_bounds__(256) cheb_deriv_kernel(const double *rr, const double *wy, int Q2, int nn, double w,
                                                          int npan, double2 *out)
 {
-    __shared__ double fv[16][5];
+    __shared__ double fv[16][5], cv[16][5];
     const int p = blockIdx.x, t = threadIdx.x, k = t >> 4, g = t & 15;
     const double cen = (p + 0.5) * w, hh = 0.5 * w;
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -1248,10 +1114,18 @@ __global__ void __launch_bounds__(256) cheb_deriv_kernel(const double *rr, const
             for (int i = 0; i < 5; ++i) c[i] = fma(fv[q][i], cq, c[i]);
         }
         const double sc = (t == 0 ? 1.0 : 2.0) / nn;
+#pragma unroll
+        for (int i = 0; i < 5; ++i) cv[t][i] = c[i] * sc;
+    }
+    __syncthreads();
+    if (t < nn) {
+        double c[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) c[i] = to_power(&cv[0][i], 5, t);
         const size_t tab = (size_t)npan * nn, o = (size_t)p * nn + t;
-        out[o] = make_double2(c[0] * sc, c[1] * sc);
-        out[tab + o] = make_double2(c[2] * sc, c[3] * sc);
-        out[2 * tab + o] = make_double2(c[4] * sc, 0.0);
+        out[o] = make_double2(c[0], c[1]);
+        out[tab + o] = make_double2(c[2], c[3]);
+        out[2 * tab + o] = make_double2(c[4], 0.0);
     }
 }
 }  // namespace
@@ -1276,7 +1150,8 @@ __global__ void e_table_kernel(const double *tt, int Q, int Mlast, double qs, do
         double sv, cv;
         sincos(q * tt[m], &sv, &cv);
         E[i] = make_double2(cv, sv);
-        if (Ef) Ef[i] = make_float2((float)cv, (float)sv);
+        // float copy by node, [m][b] for b <= Mlast/2 (the coefficients formed)
+        if (Ef && b <= Mlast / 2) Ef[(size_t)m * GF_EF_ROW(Mlast) + b] = make_float2((float)cv, (float)sv);
     }
 }
 
@@ -1394,7 +1269,7 @@ cudaError_t gf_launch_e_table(const double *tt, int Q, int Mlast, double qs, dou
 cudaError_t gf_launch_cheb_table(int dim, const double *rr, const double2 *B, const double *P0, const double *P1, int Q,
                                  int npan, int deg, double w, double2 *out, float2 *outf, cudaStream_t s)
 {
-    if (deg + 1 > 16 || npan < 1) return cudaErrorInvalidValue;
+    if (deg != GF_HDEG || npan < 1) return cudaErrorInvalidValue;
     if (dim == 3)
         cheb_table_kernel<3><<<npan, 256, 0, s>>>(rr, B, P0, P1, Q, deg + 1, w, out, outf);
     else
