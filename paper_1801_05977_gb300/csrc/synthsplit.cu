@@ -12,9 +12,14 @@
 // a store), the X' nodes' phases E are the same address for a whole warp, and
 // neighbouring columns read neighbouring panels of the h(s) table.  A thread
 // keeps the X' sums of eight b: per node one load of A and four of E (two b
-// each) against sixteen FMAs.  The columns whose coefficients need double
-// went, when they shared the float columns' CTAs, to 128 threads of 256 and to
-// one SM per eight columns; as units of their own they spread over the chip.
+// each) against sixteen FMAs.
+//
+// What bounds it: issue (the X' sums, 15 multiply-adds on a table entry each for h(s), the
+// transforms), about a third of the slots used; the store is 0.3 GB of the 1.5 ms below.
+// Before, a CTA held 8 columns by [column][b]: half its threads had no item, each lane read its
+// own line of E, the double set-up ran on 8 lanes of a warp and the double columns held
+// their CTA up.  Batched, 64 pairs with 0.5 <= k <= 5 on 32^2 x 64 to 256^2 x 64: 5.86 -> 1.47 ms.
+// One plan (cold): 128 x 128 x 64 85 -> 32 us, Maxwell 256 x 256 x 64 319 -> 125 us.
 #include <stdint.h>
 
 #include "gf_internal.cuh"
