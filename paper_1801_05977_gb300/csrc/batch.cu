@@ -142,7 +142,6 @@ static gf_status batch_eval_setup(gf_batch_t b, const double *x, const int64_t *
     b->eb.nf = b->nf;
     b->eb.grid_near = pre[b->np] < b->nsm * 16 ? (pre[b->np] > 0 ? pre[b->np] : 1) : b->nsm * 16;
     b->eb.scatter_per_pair = 2;
-    b->eb.near_lists = b->nf == 1;
     b->eb.grid_scatter = b->np * 2 < b->nsm * 4 ? b->np * 2 : b->nsm * 4;
     b->eb.block_far = b->tune.far_block;
     b->eb.grid_far = b->nsm * b->tune.far_per_sm * 128 / b->tune.far_block;

@@ -212,44 +212,118 @@ __device__ __forceinline__ int far_bucket(double z, double c)
 // 3D near kernel.  NF = 1: Helmholtz (field L_d).  NF = 7: Maxwell
 // (fields 0..5 = (delta_pq - c^p c^q/k^2) L_d, field 6 = L_d).
 // R = storage/accumulation type of the grid (double: GF_FP64, float: split).
+//
+// What the near branch is made of at one target (finite, |x3| <= c; Algorithm 2,
+// calculation step): the stencil and the phase (near_lane), the tensor cubic
+// interpolation of the stored grid, the lift (store_near), and within 2 eps of
+// a source the singular part (near_sing), added to the stored entries.  The
+// far-region grid shares all but the last.
 // ---------------------------------------------------------------------------
-// The near branch at one target i (valid, finite, |x_last| <= c): cell
-// reduction, tensor cubic interpolation of the stored grid, phases and the
-// singular part (Algorithm 2, calculation step).
+
+// One target's stencil: offset of its first node in the grid, position within
+// the cell on each axis, e^{i alpha . x} and what the exceptions need.
+template <typename R>
+struct NearLane {
+    int64_t off;     // (i3 P2 + i2) P1 + i1
+    R f1, f2, f3;
+    R lx, ly;        // e^{i alpha . x} = e^{i alpha . t} e^{i 2 pi <alpha . m>}
+    int i3n;         // x3 stencil node (near grid)
+    bool neg, sing;  // x3 < 0; within 2 eps of a source (a little more)
+};
+
+// Node floor(u) and d = u - 1/2 - floor(u) in [-1/2, 1/2] from v = u - 1/2: the sum
+// with 1.5 2^52 rounds v to an integer and leaves it (modulo 2^32) in the low
+// word.  Where u is an integer either neighbour may be taken, the interpolant is
+// the node's value for both.
+__device__ __forceinline__ int node_of(double v, double &d)
+{
+    const double w = v + 6755399441055744.0;
+    d = v - (w - 6755399441055744.0);
+    return __double2loint(w);
+}
+
+// Five double operations an axis and five for the phase, against 23 and 60: the
+// double pipe takes a warp instruction in 16 cycles, and bounds the near kernels of
+// both precisions.  The stencil coordinate comes from x itself (the in-plane
+// axes are periodic in powers of two: the node is its low bits), the lift from
+// alpha . x, both good to a rounding of x.
+template <typename R, bool FGRID>
+__device__ __forceinline__ NearLane<R> near_lane(const EvalArgs &a, double x1, double x2, double x3, bool mirror)
+{
+    NearLane<R> L;
+    const GatherArgs &g = a.ga;
+    double d1, d2, d3;
+    const int i1 = node_of(fma(x1, FGRID ? g.fih1 : g.ih1, FGRID ? g.fo1 : g.o1), d1) & ((FGRID ? a.fM1 : a.M1) - 1);
+    const int i2 = node_of(fma(x2, FGRID ? g.fih1 : g.ih2, FGRID ? g.fo1 : g.o2), d2) & ((FGRID ? a.fM2 : a.M2) - 1);
+    int i3;
+    if (FGRID) {
+        // planes are not padded: the stencil planes are i3 .. i3 + 3
+        const double v = fma(fabs(x3), g.fihz, g.foz);
+        const int n = node_of(v, d3), nc = min(max(n, 1), a.fNZ - 3);
+        if (nc != n) d3 = v - (double)nc;
+        L.i3n = nc;
+        i3 = nc - 1;
+    } else {
+        // stored planes from Q3lo: a Helmholtz grid (even in x3) holds x3 >= -h3 only
+        // and is read at |x3|; so is a Maxwell grid that keeps the odd fields' Nyquist
+        // planes (nyqgrid), otherwise it holds the slab |x3| <= c
+        const double v = fma(mirror ? fabs(x3) : x3, g.ih3, g.o3);
+        const int n = node_of(v, d3), nc = min(max(n, 0), a.M3 - 1);
+        if (nc != n) d3 = v - (double)nc;
+        L.i3n = nc;
+        i3 = nc - a.Q3lo;
+    }
+    L.off = FGRID ? ((int64_t)i3 * a.fP2 + i2) * a.fP1 + i1 : ((int64_t)i3 * a.P2 + i2) * a.P1 + i1;
+    L.f1 = (R)d1 + (R)0.5;
+    L.f2 = (R)d2 + (R)0.5;
+    L.f3 = (R)d3 + (R)0.5;
+    double ph = fma(x1, g.al1, x2 * g.al2);
+    ph -= rint(ph);
+    if (sizeof(R) == 4) {
+        float s, c;
+        sincospif(2.0f * (float)ph, &s, &c);
+        L.lx = (R)c;
+        L.ly = (R)s;
+    } else {
+        double s, c;
+        sincospi(2.0 * ph, &s, &c);
+        L.lx = (R)c;
+        L.ly = (R)s;
+    }
+    L.neg = x3 < 0.0;
+    L.sing = false;
+    if (!FGRID) {
+        const float t1 = fmaf((float)i1 + (float)L.f1, g.h1, -(float)GF_PI), t2 = fmaf((float)i2 + (float)L.f2, g.h2, -(float)GF_PI);
+        const float t3 = (float)x3;
+        L.sing = t1 * t1 + t2 * t2 + t3 * t3 < g.rs2;
+    }
+    return L;
+}
+
+// (a b) in float, each part by Kahan's two-product difference: 1.5 roundings of the
+// result, as a product in double rounded once, without the double pipe.
+__device__ __forceinline__ float2 cmul_kahan(float2 a, float2 b)
+{
+    const float w = a.y * b.y, v = -a.y * b.x;
+    return make_float2(fmaf(a.x, b.x, -w) - fmaf(a.y, b.y, -w), fmaf(a.x, b.y, -v) - fmaf(-a.y, b.x, -v));
+}
+__device__ __forceinline__ float2 lift_mul(float2 a, float2 b) { return cmul_kahan(a, b); }
+__device__ __forceinline__ double2 lift_mul(double2 a, double2 b) { return cmul(a, b); }
+
+// Tensor cubic interpolation by one thread: P1, P2 the grid's padded extents.
 template <typename R, int NF>
-__device__ __forceinline__ void near_point(const EvalArgs &a, int64_t i, double x1, double x2, double x3, double ih1,
-                                           double ih2, double ih3)
+__device__ __forceinline__ void gather_lane(const void *grid, int P1, int P2, const NearLane<R> &L, const R w1[4], const R w2[4],
+                                            const R w3[4], R acc[NF][2])
 {
     typedef typename cplx_t<R>::T C;
-    const C *G = reinterpret_cast<const C *>(a.grid);
-    const int ne = n_entries(a.which);
-    C *o = reinterpret_cast<C *>(a.out) + i * ne;
-    const bool only_L = NF == 1 && a.which == GF_OUT_LD;
-    double t1, m1, t2, m2;
-    reduce_period(x1, t1, m1);
-    reduce_period(x2, t2, m2);
-    double f1, f2, f3;
-    int i1 = stencil_origin(t1, -GF_PI, a.h1, ih1, a.M1, f1);
-    int i2 = stencil_origin(t2, -GF_PI, a.h2, ih2, a.M2, f2);
-    // stored planes from Q3lo: a Helmholtz grid (even in x3) holds x3 >= -h3 only
-    // and is read at |x3|; so is a Maxwell grid that keeps the odd fields' Nyquist
-    // planes (nyqgrid), otherwise it holds the slab |x3| <= c
-    const bool mirror = NF == 1 || a.nyqgrid != nullptr;
-    const int i3n = stencil_origin(mirror ? fabs(x3) : x3, -a.ct, a.h3, ih3, a.M3, f3);
-    const int i3 = i3n - a.Q3lo;
-    // weights in the grid's precision (f itself is formed in double)
-    R w1[4], w2[4], w3[4];
-    lagrange4<R>((R)f1, w1);
-    lagrange4<R>((R)f2, w2);
-    lagrange4<R>((R)f3, w3);
-    R acc[NF][2];
+    const C *G = reinterpret_cast<const C *>(grid) + L.off * NF;
 #pragma unroll
     for (int e = 0; e < NF; ++e) acc[e][0] = acc[e][1] = (R)0;
 #pragma unroll
     for (int d3 = 0; d3 < 4; ++d3) {
 #pragma unroll
         for (int d2 = 0; d2 < 4; ++d2) {
-            const C *row = G + (((size_t)(i3 + d3) * a.P2 + (i2 + d2)) * a.P1 + i1) * NF;
+            const C *row = G + ((size_t)d3 * P2 + d2) * P1 * NF;
             const R w23 = w3[d3] * w2[d2];
 #pragma unroll
             for (int e = 0; e < NF; ++e) {
@@ -263,202 +337,364 @@ __device__ __forceinline__ void near_point(const EvalArgs &a, int64_t i, double 
                 acc[e][0] = fma(w23, sr, acc[e][0]);
                 acc[e][1] = fma(w23, si, acc[e][1]);
             }
-        }
-    }
-    if (NF > 1 && a.nyqgrid != nullptr && x3 < 0.0) {
-        // The stencil of x3 < 0 is the mirror of the one read at |x3| (nodes
-        // a' = i3n - 1 .. i3n + 2 <-> M3 - a').  Even fields: the same values.  Odd
-        // fields (4: xz, 5: yz): L(M3 - a') = -L(a') + 2 (-1)^(M3/2 + a') P(t), so
-        // the interpolant is -acc + 2 (-1)^(M3/2) (sum_d w3_d (-1)^(a'_d)) P(t),
-        // P interpolated bicubically from the Nyquist planes.
-        R sgn = w3[0] - w3[1] + w3[2] - w3[3];
-        if (((i3n - 1) ^ (a.M3 >> 1)) & 1) sgn = -sgn;
-        const C *NG = reinterpret_cast<const C *>(a.nyqgrid);
-        R pr[2] = {0, 0}, pi[2] = {0, 0};
-#pragma unroll
-        for (int d2 = 0; d2 < 4; ++d2) {
-            const C *row = NG + ((size_t)(i2 + d2) * a.P1 + i1) * 2;
-            R s4r = 0, s4i = 0, s5r = 0, s5i = 0;
-#pragma unroll
-            for (int d1 = 0; d1 < 4; ++d1) {
-                const C g4 = __ldg(row + 2 * d1), g5 = __ldg(row + 2 * d1 + 1);
-                s4r = fma(w1[d1], g4.x, s4r);
-                s4i = fma(w1[d1], g4.y, s4i);
-                s5r = fma(w1[d1], g5.x, s5r);
-                s5i = fma(w1[d1], g5.y, s5i);
-            }
-            pr[0] = fma(w2[d2], s4r, pr[0]);
-            pi[0] = fma(w2[d2], s4i, pi[0]);
-            pr[1] = fma(w2[d2], s5r, pr[1]);
-            pi[1] = fma(w2[d2], s5i, pi[1]);
-        }
-        const R two_s = (R)2 * sgn;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            acc[4 + q][0] = fma(two_s, pr[q], -acc[4 + q][0]);
-            acc[4 + q][1] = fma(two_s, pi[q], -acc[4 + q][1]);
-        }
-    }
-
-    // lift = e^{i alpha.t} e^{i 2 pi <alpha.m>}; G = lift L + e^{i 2pi<alpha.m>} Phi Y (K = L + F, F = e^{-i alpha.t} Phi Y).
-    // Split plans: the fractional part in double, the two phases in float.
-    double2 lat, lift;
-    float2 latf = make_float2(0.f, 0.f), liftf = make_float2(0.f, 0.f);
-    if (sizeof(R) == 4) {
-        double ph = a.a1 * m1 + a.a2 * m2;
-        ph -= rint(ph);
-        float sl, cl, sa, ca;
-        sincospif(2.0f * (float)ph, &sl, &cl);
-        sincosf((float)a.a1 * (float)t1 + (float)a.a2 * (float)t2, &sa, &ca);
-        latf = make_float2(cl, sl);
-        liftf = cmulf(make_float2(ca, sa), latf);
-        lat = make_double2(cl, sl);
-        lift = make_double2(liftf.x, liftf.y);
-    } else {
-        lat = lattice_phase(a.a1, m1, a.a2, m2);
-        double sa, ca;
-        sincos(a.a1 * t1 + a.a2 * t2, &sa, &ca);
-        lift = cmul(make_double2(ca, sa), lat);
-    }
-    double r = sqrt(t1 * t1 + t2 * t2 + x3 * x3);
-    bool sing = r < 2.0 * a.eps;
-    double2 PhiY = make_double2(0, 0), dPhi = make_double2(0, 0), d2Phi = make_double2(0, 0);
-    if (sing) {
-        // Phi(r) = e^{ikr}/(4 pi r) Y_eps(r) and its r-derivatives (Sec. 3.2, Sec. 4)
-        double sk, ck;
-        sincos(a.k * r, &sk, &ck);
-        double ir = 1.0 / r;
-        double2 g0 = make_double2(ck * ir * (0.25 / GF_PI), sk * ir * (0.25 / GF_PI));
-        double s = (r - a.eps) / a.eps;
-        double Y0 = 1.0 - smooth8(s);
-        PhiY = cscale(g0, Y0);
-        if (NF > 1) {
-            double Y1 = -smooth8_d1(s) / a.eps;
-            double Y2 = -smooth8_d2(s) / (a.eps * a.eps);
-            double2 L1 = make_double2(-ir, a.k);                  // ik - 1/r
-            double2 g1 = cmul(g0, L1);
-            double2 L2 = cmul(L1, L1);
-            L2.x += ir * ir;
-            double2 g2 = cmul(g0, L2);
-            dPhi = cadd(cscale(g1, Y0), cscale(g0, Y1));
-            d2Phi = cadd(cadd(cscale(g2, Y0), cscale(g1, 2.0 * Y1)), cscale(g0, Y2));
-        }
-    }
-    if (NF == 1) {
-        double2 L = make_double2((double)acc[0][0], (double)acc[0][1]);
-        if (only_L) {
-            store_out(o, L);
-            return;
-        }
-        if (sizeof(R) == 4) {
-            // split: the combination in float (the singular part was formed in double)
-            const float2 v = cmulf(liftf, make_float2((float)acc[0][0], (float)acc[0][1]));
-            const float2 u = sing ? cmulf(latf, make_float2((float)PhiY.x, (float)PhiY.y)) : make_float2(0.f, 0.f);
-            reinterpret_cast<float2 *>(o)[0] = make_float2(v.x + u.x, v.y + u.y);
-            return;
-        }
-        double2 v = cadd(cmul(lift, L), cmul(lat, PhiY));
-        store_out(o, v);
-    } else {
-        const double ik2 = 1.0 / (a.k * a.k);
-        const double xv[3] = {t1, t2, x3};
-        const int PP[6] = {0, 1, 2, 0, 0, 1}, QQ[6] = {0, 1, 2, 1, 2, 2};
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-            double2 L = make_double2((double)acc[e][0], (double)acc[e][1]);
-            double2 v = cmul(lift, L);
-            if (sing) {
-                double ir = 1.0 / r;
-                double xp = xv[PP[e]] * ir, xq = xv[QQ[e]] * ir;
-                double dl = PP[e] == QQ[e] ? 1.0 : 0.0;
-                // delta_pq Phi + k^-2 [Phi'' xp xq + (Phi'/r)(delta_pq - xp xq)]
-                double2 s = cadd(cscale(d2Phi, xp * xq), cscale(dPhi, ir * (dl - xp * xq)));
-                s = cscale(s, ik2);
-                if (dl != 0.0) s = cadd(s, PhiY);
-                v = cadd(v, cmul(lat, s));
-            }
-            store_out(o + e, v);
-        }
-        if (a.which == GF_OUT_MAXWELL7) {
-            double2 L = make_double2((double)acc[6][0], (double)acc[6][1]);
-            store_out(o + 6, cadd(cmul(lift, L), cmul(lat, PhiY)));
         }
     }
 }
 
-// Far-region grid at one target i (valid, finite, c < |x3| <= fzmax): the same
-// cell reduction as the near branch, tensor cubic interpolation of the far
-// planes (in z from fz0 with the stencil origin clamped to the last full
-// interval), and the lift e^{i alpha.t} e^{i 2 pi <alpha.m>}; the Maxwell xz and
-// yz entries change sign with x3.  No singular part: |x3| > c >= 2 eps.
-template <typename R, int NF>
-__device__ __forceinline__ void far_grid_point(const EvalArgs &a, int64_t i, double x1, double x2, double x3)
+// The stencil of x3 < 0 on a half grid is the mirror of the one read at |x3| (nodes
+// a' = i3n - 1 .. i3n + 2 <-> M3 - a').  Even fields: the same values.  Odd
+// fields (4: xz, 5: yz): L(M3 - a') = -L(a') + 2 (-1)^(M3/2 + a') P(t), so
+// the interpolant is -acc + 2 (-1)^(M3/2) (sum_d w3_d (-1)^(a'_d)) P(t),
+// P interpolated bicubically from the Nyquist planes.  The factor of P:
+template <typename R>
+__device__ __forceinline__ R nyq_factor(const EvalArgs &a, int i3n, const R w3[4])
+{
+    const R sgn = w3[0] - w3[1] + w3[2] - w3[3];
+    return (((i3n - 1) ^ (a.M3 >> 1)) & 1) ? (R)-2 * sgn : (R)2 * sgn;
+}
+
+template <typename R>
+__device__ __forceinline__ void nyq_lane(const EvalArgs &a, const NearLane<R> &L, const R w1[4], const R w2[4], const R w3[4],
+                                         R acc[][2])
 {
     typedef typename cplx_t<R>::T C;
-    const C *G = reinterpret_cast<const C *>(a.fargrid);
+    const C *NG = reinterpret_cast<const C *>(a.nyqgrid);
+    const int i21 = (int)L.off - (L.i3n - a.Q3lo) * a.P2 * a.P1;
+    R pr[2] = {0, 0}, pi[2] = {0, 0};
+#pragma unroll
+    for (int d2 = 0; d2 < 4; ++d2) {
+        const C *row = NG + ((size_t)i21 + (size_t)d2 * a.P1) * 2;
+        R s4r = 0, s4i = 0, s5r = 0, s5i = 0;
+#pragma unroll
+        for (int d1 = 0; d1 < 4; ++d1) {
+            const C g4 = __ldg(row + 2 * d1), g5 = __ldg(row + 2 * d1 + 1);
+            s4r = fma(w1[d1], g4.x, s4r);
+            s4i = fma(w1[d1], g4.y, s4i);
+            s5r = fma(w1[d1], g5.x, s5r);
+            s5i = fma(w1[d1], g5.y, s5i);
+        }
+        pr[0] = fma(w2[d2], s4r, pr[0]);
+        pi[0] = fma(w2[d2], s4i, pi[0]);
+        pr[1] = fma(w2[d2], s5r, pr[1]);
+        pi[1] = fma(w2[d2], s5i, pi[1]);
+    }
+    const R two_s = nyq_factor<R>(a, L.i3n, w3);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        acc[4 + q][0] = fma(two_s, pr[q], -acc[4 + q][0]);
+        acc[4 + q][1] = fma(two_s, pi[q], -acc[4 + q][1]);
+    }
+}
+
+// Entries of target i: lift L (the remainder alone for GF_OUT_LD); the Maxwell xz and yz
+// entries of the far-region grid change sign with x3.
+template <typename R, int NF, bool FGRID>
+__device__ __forceinline__ void store_near(const EvalArgs &a, int64_t i, const NearLane<R> &L, const R acc[NF][2])
+{
+    typedef typename cplx_t<R>::T C;
     const int ne = n_entries(a.which);
     C *o = reinterpret_cast<C *>(a.out) + i * ne;
+    const C lift = cmk(L.lx, L.ly);
+    if (NF == 1) {
+        const C v = cmk(acc[0][0], acc[0][1]);
+        o[0] = a.which == GF_OUT_LD ? v : lift_mul(lift, v);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 7; ++e) {
+            C v = lift_mul(lift, cmk(acc[e < NF ? e : 0][0], acc[e < NF ? e : 0][1]));
+            if (FGRID && (e == 4 || e == 5) && L.neg) v = cmk(-v.x, -v.y);
+            if (e < ne) o[e] = v;
+        }
+    }
+}
+
+// *o += v, rounded once (the caller's own entry).
+__device__ __forceinline__ void add_near(double2 *o, double2 v) { *o = cadd(*o, v); }
+__device__ __forceinline__ void add_near(float2 *o, double2 v)
+{
+    const float2 u = *o;
+    *o = make_float2((float)((double)u.x + v.x), (float)((double)u.y + v.y));
+}
+
+// The singular part at target i, e^{i 2pi<alpha.m>} Phi Y (G = lift L + that, K = L + F, F =
+// e^{-i alpha.t} Phi Y) and for Maxwell its derivatives, added to the stored entries.
+// Not forced inline: one target in sixteen of a uniform slab comes here.
+template <typename R, int NF>
+__device__ __noinline__ void near_sing(const EvalArgs &a, int64_t i)
+{
+    typedef typename cplx_t<R>::T C;
+    const int ne = n_entries(a.which);
+    C *o = reinterpret_cast<C *>(a.out) + i * ne;
+    const double x3 = a.x[3 * i + 2];
     double t1, m1, t2, m2;
-    reduce_period(x1, t1, m1);
-    reduce_period(x2, t2, m2);
-    double f1, f2, f3;
-    const int i1 = stencil_origin(t1, -GF_PI, a.fh1, 1.0 / a.fh1, a.fM1, f1);
-    const int i2 = stencil_origin(t2, -GF_PI, a.fh2, 1.0 / a.fh2, a.fM2, f2);
-    // planes are not padded: the stencil planes are i0 - 1 .. i0 + 2, i0 <= fNZ - 3
-    const int i3 = stencil_origin(fabs(x3), a.fz0, a.fhz, 1.0 / a.fhz, a.fNZ - 2, f3) - 1;
-    R w1[4], w2[4], w3[4];
-    lagrange4<R>((R)f1, w1);
-    lagrange4<R>((R)f2, w2);
-    lagrange4<R>((R)f3, w3);
-    R acc[NF][2];
+    reduce_period(a.x[3 * i], t1, m1);
+    reduce_period(a.x[3 * i + 1], t2, m2);
+    const double r = sqrt(t1 * t1 + t2 * t2 + x3 * x3);
+    if (!(r < 2.0 * a.eps)) return;
+    const double2 lat = lattice_phase(a.a1, m1, a.a2, m2);
+    // Phi(r) = e^{ikr}/(4 pi r) Y_eps(r) and its r-derivatives (Sec. 3.2, Sec. 4)
+    double sk, ck;
+    sincos(a.k * r, &sk, &ck);
+    const double ir = 1.0 / r;
+    const double2 g0 = make_double2(ck * ir * (0.25 / GF_PI), sk * ir * (0.25 / GF_PI));
+    const double s = (r - a.eps) / a.eps;
+    const double Y0 = 1.0 - smooth8(s);
+    const double2 PhiY = cscale(g0, Y0);
+    if (NF == 1) {
+        add_near(o, cmul(lat, PhiY));
+        return;
+    }
+    const double Y1 = -smooth8_d1(s) / a.eps;
+    const double Y2 = -smooth8_d2(s) / (a.eps * a.eps);
+    const double2 L1 = make_double2(-ir, a.k);                  // ik - 1/r
+    const double2 g1 = cmul(g0, L1);
+    double2 L2 = cmul(L1, L1);
+    L2.x += ir * ir;
+    const double2 g2 = cmul(g0, L2);
+    const double2 dPhi = cadd(cscale(g1, Y0), cscale(g0, Y1));
+    const double2 d2Phi = cadd(cadd(cscale(g2, Y0), cscale(g1, 2.0 * Y1)), cscale(g0, Y2));
+    const double ik2 = 1.0 / (a.k * a.k);
+    const double xv[3] = {t1, t2, x3};
+    const int PP[6] = {0, 1, 2, 0, 0, 1}, QQ[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
-    for (int e = 0; e < NF; ++e) acc[e][0] = acc[e][1] = (R)0;
+    for (int e = 0; e < 6; ++e) {
+        const double xp = xv[PP[e]] * ir, xq = xv[QQ[e]] * ir;
+        const double dl = PP[e] == QQ[e] ? 1.0 : 0.0;
+        // delta_pq Phi + k^-2 [Phi'' xp xq + (Phi'/r)(delta_pq - xp xq)]
+        double2 v = cadd(cscale(d2Phi, xp * xq), cscale(dPhi, ir * (dl - xp * xq)));
+        v = cscale(v, ik2);
+        if (dl != 0.0) v = cadd(v, PhiY);
+        add_near(o + e, cmul(lat, v));
+    }
+    if (a.which == GF_OUT_MAXWELL7) add_near(o + 6, cmul(lat, PhiY));
+}
+
+// One target by one thread (evaluations without list scratch).
+template <typename R, int NF, bool FGRID>
+__device__ __forceinline__ void near_point(const EvalArgs &a, int64_t i, double x1, double x2, double x3)
+{
+    const NearLane<R> L = near_lane<R, FGRID>(a, x1, x2, x3, NF == 1 || a.nyqgrid != nullptr);
+    R w1[4], w2[4], w3[4], acc[NF][2];
+    lagrange4<R>(L.f1, w1);
+    lagrange4<R>(L.f2, w2);
+    lagrange4<R>(L.f3, w3);
+    gather_lane<R, NF>(FGRID ? a.fargrid : a.grid, FGRID ? a.fP1 : a.P1, FGRID ? a.fP2 : a.P2, L, w1, w2, w3, acc);
+    if (NF > 1 && !FGRID && a.nyqgrid != nullptr && L.neg) nyq_lane<R>(a, L, w1, w2, w3, acc);
+    store_near<R, NF, FGRID>(a, i, L, acc);
+    if (L.sing && a.which != GF_OUT_LD) near_sing<R, NF>(a, i);
+}
+
+// ---------------------------------------------------------------------------
+// Listed targets, 32 at a time by one warp.
+//
+// Read by its own thread, a target's stencil costs 64 NF loads of which every lane
+// touches another cache line: the L1 takes 32 cycles for each (14,300 a warp with
+// seven fields in float; 0.8 of the kernel's time).  Here the lanes that take one row of a
+// stencil are neighbours: one field, four lanes a target (x1 nodes), eight targets a load;
+// seven fields, 28 lanes (node, field), one target a load.  The products w3 w2 and
+// the weights w1 come from the warp's shared memory, the sums over x1 by
+// shuffles, and with seven fields the lanes write a target's entries side by side.
+// (Seven fields in double stay with one thread a target: there the double pipe
+// is the limit, and 28 lanes of 32 and the shuffled sums would cost more of it.)
+// The targets next to a source wait in the warp's queue until a full warp of
+// them is there: most warps hold one or two, and would all pay for the singular part.
+// ---------------------------------------------------------------------------
+constexpr int NEAR_WARPS = 4;
+template <typename R> constexpr int near_ws() { return sizeof(R) == 4 ? 20 : 22; }  // w23 [16], w1 [4] (and bank padding)
+
+struct SingItem {
+    int pair, i;
+};
+template <typename R, int NF>
+struct NearWarp {
+    R w[sizeof(R) == 8 && NF > 1 ? 1 : 32][near_ws<R>()];
+    SingItem q[64];
+};
+
+template <typename R>
+__device__ __forceinline__ void gather_quads(const void *grid, int P1, int P2, int64_t off, const R (*w)[near_ws<R>()], R acc[1][2])
+{
+    typedef typename cplx_t<R>::T C;
+    const int lane = threadIdx.x & 31, d1 = lane & 3;
+    const size_t P12 = (size_t)P1 * P2;
+    acc[0][0] = acc[0][1] = (R)0;
+#pragma unroll 1
+    for (int p = 0; p < 4; ++p) {
+        const int src = p * 8 + (lane >> 2);
+        const C *g = reinterpret_cast<const C *>(grid) + __shfl_sync(0xffffffffu, off, src) + d1;
+        const R *ws = w[src];
+        R ax = 0, ay = 0;
 #pragma unroll
-    for (int d3 = 0; d3 < 4; ++d3) {
+        for (int d3 = 0; d3 < 4; ++d3)
 #pragma unroll
-        for (int d2 = 0; d2 < 4; ++d2) {
-            const C *row = G + (((size_t)(i3 + d3) * a.fP2 + (i2 + d2)) * a.fP1 + i1) * NF;
-            const R w23 = w3[d3] * w2[d2];
+            for (int d2 = 0; d2 < 4; ++d2) {
+                const C v = __ldg(g + d3 * P12 + d2 * P1);
+                const R w23 = ws[d3 * 4 + d2];
+                ax = fma(w23, v.x, ax);
+                ay = fma(w23, v.y, ay);
+            }
+        const R w1 = ws[16 + d1];
+        ax *= w1;
+        ay *= w1;
+        ax += __shfl_xor_sync(0xffffffffu, ax, 1);
+        ay += __shfl_xor_sync(0xffffffffu, ay, 1);
+        ax += __shfl_xor_sync(0xffffffffu, ax, 2);
+        ay += __shfl_xor_sync(0xffffffffu, ay, 2);
+        const R rx = __shfl_sync(0xffffffffu, ax, (lane & 7) * 4), ry = __shfl_sync(0xffffffffu, ay, (lane & 7) * 4);
+        if ((lane >> 3) == p) {
+            acc[0][0] = rx;
+            acc[0][1] = ry;
+        }
+    }
+}
+
+// Seven float fields: target after target, entries written by lanes 0 .. 6.
+template <bool FGRID>
+__device__ __forceinline__ void gather_rows(const EvalArgs &a, int i, int cnt, const NearLane<float> &L, float nyqf,
+                                            const float (*w)[near_ws<float>()])
+{
+    const int lane = threadIdx.x & 31, ne = n_entries(a.which), d1 = lane < 28 ? lane / 7 : 3;
+    const int P1 = FGRID ? a.fP1 : a.P1, P2 = FGRID ? a.fP2 : a.P2;
+    const size_t s2 = (size_t)P1 * 7, s3 = s2 * P2;
+    const float2 *G = reinterpret_cast<const float2 *>(FGRID ? a.fargrid : a.grid) + (lane < 28 ? lane : 27);
+    const bool half = !FGRID && a.nyqgrid != nullptr;
+    const unsigned negs = __ballot_sync(0xffffffffu, L.neg);
+    const int P12 = P1 * P2;
+#pragma unroll 1
+    for (int t = 0; t < cnt; ++t) {
+        const int64_t off = __shfl_sync(0xffffffffu, L.off, t);
+        const int it = __shfl_sync(0xffffffffu, i, t);
+        const float lx = __shfl_sync(0xffffffffu, L.lx, t), ly = __shfl_sync(0xffffffffu, L.ly, t);
+        const float2 *g = G + off * 7;
+        const float *ws = w[t];
+        float ax = 0.f, ay = 0.f;
 #pragma unroll
-            for (int e = 0; e < NF; ++e) {
-                R sr = 0, si = 0;
+        for (int d3 = 0; d3 < 4; ++d3)
 #pragma unroll
-                for (int d1 = 0; d1 < 4; ++d1) {
-                    C g = __ldg(row + d1 * NF + e);
-                    sr = fma(w1[d1], g.x, sr);
-                    si = fma(w1[d1], g.y, si);
-                }
-                acc[e][0] = fma(w23, sr, acc[e][0]);
-                acc[e][1] = fma(w23, si, acc[e][1]);
+            for (int d2 = 0; d2 < 4; ++d2) {
+                const float2 v = __ldg(g + d3 * s3 + d2 * s2);
+                const float w23 = ws[d3 * 4 + d2];
+                ax = fmaf(w23, v.x, ax);
+                ay = fmaf(w23, v.y, ay);
+            }
+        const float w1 = ws[16 + d1];
+        ax *= w1;
+        ay *= w1;
+        ax += __shfl_down_sync(0xffffffffu, ax, 14);
+        ay += __shfl_down_sync(0xffffffffu, ay, 14);
+        ax += __shfl_down_sync(0xffffffffu, ax, 7);
+        ay += __shfl_down_sync(0xffffffffu, ay, 7);
+        const bool neg = (negs >> t) & 1;
+        if (half && neg) {
+            // the Nyquist planes' stencil: lane = (d2, d1, field), and the sum over the nodes
+            const int i21 = (int)off % P12;
+            const float nf = __shfl_sync(0xffffffffu, nyqf, t);
+            const float *wt = ws + 16;
+            const float2 v = __ldg(reinterpret_cast<const float2 *>(a.nyqgrid) +
+                                   ((size_t)i21 + (size_t)(lane >> 3) * P1 + ((lane >> 1) & 3)) * 2 + (lane & 1));
+            // w2[d2] = sum over d3 of w3[d3] w2[d2] (the w3 sum to 1)
+            const int q2 = lane >> 3;
+            const float w2 = (ws[q2] + ws[4 + q2]) + (ws[8 + q2] + ws[12 + q2]);
+            const float ww = w2 * wt[(lane >> 1) & 3];
+            float px = ww * v.x, py = ww * v.y;
+#pragma unroll
+            for (int o = 2; o < 32; o <<= 1) {
+                px += __shfl_xor_sync(0xffffffffu, px, o);
+                py += __shfl_xor_sync(0xffffffffu, py, o);
+            }
+            if (lane == 4 || lane == 5) {
+                ax = fmaf(nf, px, -ax);
+                ay = fmaf(nf, py, -ay);
             }
         }
-    }
-    if (sizeof(R) == 4) {
-        double ph = a.a1 * m1 + a.a2 * m2;
-        ph -= rint(ph);
-        float sl, cl, sa, ca;
-        sincospif(2.0f * (float)ph, &sl, &cl);
-        sincosf((float)a.a1 * (float)t1 + (float)a.a2 * (float)t2, &sa, &ca);
-        const float2 lift = cmulf(make_float2(ca, sa), make_float2(cl, sl));
-        float2 *of = reinterpret_cast<float2 *>(o);
-        for (int e = 0; e < ne; ++e) {
-            const int f = NF == 1 ? 0 : (e < 6 ? e : 6);
-            float2 v = cmulf(lift, make_float2((float)acc[f][0], (float)acc[f][1]));
-            if (NF > 1 && (e == 4 || e == 5) && x3 < 0.0) v = make_float2(-v.x, -v.y);
-            of[e] = v;
-        }
-    } else {
-        const double2 lat = lattice_phase(a.a1, m1, a.a2, m2);
-        double sa, ca;
-        sincos(a.a1 * t1 + a.a2 * t2, &sa, &ca);
-        const double2 lift = cmul(make_double2(ca, sa), lat);
-        for (int e = 0; e < ne; ++e) {
-            const int f = NF == 1 ? 0 : (e < 6 ? e : 6);
-            double2 v = cmul(lift, make_double2((double)acc[f][0], (double)acc[f][1]));
-            if (NF > 1 && (e == 4 || e == 5) && x3 < 0.0) v = make_double2(-v.x, -v.y);
-            store_out(o + e, v);
+        if (lane < ne) {
+            float2 v = cmul_kahan(make_float2(lx, ly), make_float2(ax, ay));
+            if (FGRID && neg && (lane == 4 || lane == 5)) v = make_float2(-v.x, -v.y);
+            reinterpret_cast<float2 *>(a.out)[(size_t)it * ne + lane] = v;
         }
     }
+}
+
+// 32 targets (cnt of them valid): lane's target is i.  Returns whether the lane's target
+// needs the singular part.
+template <typename R, int NF, bool FGRID>
+__device__ __forceinline__ bool near_warp(const EvalArgs &a, int i, int cnt, NearWarp<R, NF> &sm)
+{
+    const int lane = threadIdx.x & 31;
+    const bool valid = lane < cnt;
+    double x1 = 0.0, x2 = 0.0, x3 = a.c;
+    if (valid) {
+        x1 = a.x[3 * (int64_t)i];
+        x2 = a.x[3 * (int64_t)i + 1];
+        x3 = a.x[3 * (int64_t)i + 2];
+    }
+    const NearLane<R> L = near_lane<R, FGRID>(a, x1, x2, x3, NF == 1 || a.nyqgrid != nullptr);
+    R w1[4], w2[4], w3[4];
+    lagrange4<R>(L.f1, w1);
+    lagrange4<R>(L.f2, w2);
+    lagrange4<R>(L.f3, w3);
+    R acc[NF][2];
+    if (sizeof(R) == 8 && NF > 1) {
+        gather_lane<R, NF>(FGRID ? a.fargrid : a.grid, FGRID ? a.fP1 : a.P1, FGRID ? a.fP2 : a.P2, L, w1, w2, w3, acc);
+        if (!FGRID && a.nyqgrid != nullptr && L.neg) nyq_lane<R>(a, L, w1, w2, w3, acc);
+        if (valid) store_near<R, NF, FGRID>(a, i, L, acc);
+        return valid && L.sing;
+    }
+    R *w = sm.w[sizeof(R) == 8 && NF > 1 ? 0 : lane];
+    __syncwarp();
+#pragma unroll
+    for (int d3 = 0; d3 < 4; ++d3)
+#pragma unroll
+        for (int d2 = 0; d2 < 4; ++d2) w[d3 * 4 + d2] = w3[d3] * w2[d2];
+#pragma unroll
+    for (int d1 = 0; d1 < 4; ++d1) w[16 + d1] = w1[d1];
+    __syncwarp();
+    if (NF == 1) {
+        gather_quads<R>(FGRID ? a.fargrid : a.grid, FGRID ? a.fP1 : a.P1, FGRID ? a.fP2 : a.P2, L.off, sm.w, acc);
+        if (valid) store_near<R, NF, FGRID>(a, i, L, acc);
+    } else if constexpr (sizeof(R) == 4 && NF > 1) {
+        gather_rows<FGRID>(a, i, cnt, L, nyq_factor<R>(a, L.i3n, w3), sm.w);
+    }
+    return valid && L.sing;
+}
+
+// A warp's queue of targets next to a source: n entries of q.
+template <typename R, int NF>
+__device__ __forceinline__ void sing_flush(const EvalArgs *args, NearWarp<R, NF> &sm, int &n)
+{
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < n) near_sing<R, NF>(args[sm.q[lane].pair], sm.q[lane].i);
+    __syncwarp();
+    if (n > 32) {
+        if (lane < n - 32) sm.q[lane] = sm.q[32 + lane];
+        __syncwarp();
+    }
+    n = n > 32 ? n - 32 : 0;
+}
+
+// Tile t of pair p's lists: the near targets' tiles, then the far-grid ones'.
+template <typename R, int NF>
+__device__ __forceinline__ void near_list_tile(const EvalArgs *args, int p, int t, int nnear, int nfg, NearWarp<R, NF> &sm, int &nq)
+{
+    const EvalArgs &a = args[p];
+    const int lane = threadIdx.x & 31, tn = (nnear + 31) >> 5;
+    if (t >= tn) {
+        const int j0 = (t - tn) * 32, cnt = min(nfg - j0, 32);
+        near_warp<R, NF, true>(a, a.near_idx[a.n - 1 - (j0 + min(lane, cnt - 1))], cnt, sm);
+        return;
+    }
+    const int j0 = t * 32, cnt = min(nnear - j0, 32);
+    const int i = a.near_idx[j0 + min(lane, cnt - 1)];
+    const bool sing = near_warp<R, NF, false>(a, i, cnt, sm) && a.which != GF_OUT_LD;
+    const unsigned m = __ballot_sync(0xffffffffu, sing);
+    if (sing) {
+        SingItem &q = sm.q[nq + __popc(m & ((1u << lane) - 1u))];
+        q.pair = p;
+        q.i = i;
+    }
+    nq += __popc(m);
+    if (nq >= 32) sing_flush<R, NF>(args, sm, nq);
 }
 
 // Append to the end of the near list, backwards (far-grid targets): the list
@@ -487,7 +723,6 @@ __device__ void near3d_tiles(const EvalArgs &a, int64_t base0, int64_t stride, i
     typedef typename cplx_t<R>::T C;
     C *out = reinterpret_cast<C *>(a.out);
     const int ne = n_entries(a.which);
-    const double ih1 = 1.0 / a.h1, ih2 = 1.0 / a.h2, ih3 = 1.0 / a.h3;
     for (int64_t base = base0; base < a.n; base += stride) {
         const int64_t i = base + threadIdx.x;
         bool valid = i < a.n;
@@ -522,7 +757,7 @@ __device__ void near3d_tiles(const EvalArgs &a, int64_t base0, int64_t stride, i
         }
         C *o = out + i * ne;
         if (fgrid) {
-            if (MODE == 0) far_grid_point<R, NF>(a, i, x1, x2, x3);
+            if (MODE == 0) near_point<R, NF, true>(a, i, x1, x2, x3);
             continue;
         }
         if (isfar) {
@@ -536,34 +771,22 @@ __device__ void near3d_tiles(const EvalArgs &a, int64_t base0, int64_t stride, i
             for (int e = 0; e < ne; ++e) o[e] = nan_c<R>();
             continue;
         }
-        if (MODE == 0) near_point<R, NF>(a, i, x1, x2, x3, ih1, ih2, ih3);
+        if (MODE == 0) near_point<R, NF, false>(a, i, x1, x2, x3);
     }
 }
 
-// Entry j of the targets listed by a MODE-1 classification pass: the near
-// targets (j < nnear) from the start of the list, then the far-grid ones from
-// its end.
+// The targets listed by a MODE-1 classification pass.
 template <typename R, int NF>
-__device__ __forceinline__ void list_point(const EvalArgs &a, int j, int nnear, double ih1, double ih2, double ih3)
+__global__ void __launch_bounds__(32 * NEAR_WARPS) near3d_list(const __grid_constant__ EvalArgs a)
 {
-    if (j < nnear) {
-        const int64_t i = a.near_idx[j];
-        near_point<R, NF>(a, i, a.x[3 * i], a.x[3 * i + 1], a.x[3 * i + 2], ih1, ih2, ih3);
-    } else {
-        const int64_t i = a.near_idx[a.n - 1 - (j - nnear)];
-        far_grid_point<R, NF>(a, i, a.x[3 * i], a.x[3 * i + 1], a.x[3 * i + 2]);
-    }
-}
-
-// The targets listed by a MODE-1 classification pass, one per thread.
-template <typename R, int NF>
-__global__ void __launch_bounds__(256) near3d_list(EvalArgs a)
-{
-    const int nnear = a.far_count[GF_NEAR_SLOT];
-    const int count = nnear + a.far_count[GF_FGRID_SLOT];
-    const double ih1 = 1.0 / a.h1, ih2 = 1.0 / a.h2, ih3 = 1.0 / a.h3;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x)
-        list_point<R, NF>(a, j, nnear, ih1, ih2, ih3);
+    __shared__ __align__(16) NearWarp<R, NF> smem[NEAR_WARPS];
+    NearWarp<R, NF> &sm = smem[threadIdx.x >> 5];
+    const int nnear = a.far_count[GF_NEAR_SLOT], nfg = a.far_count[GF_FGRID_SLOT];
+    const int tiles = ((nnear + 31) >> 5) + ((nfg + 31) >> 5);
+    int nq = 0;
+    for (int t = blockIdx.x * NEAR_WARPS + (threadIdx.x >> 5); t < tiles; t += gridDim.x * NEAR_WARPS)
+        near_list_tile<R, NF>(&a, 0, t, nnear, nfg, sm, nq);
+    if (nq) sing_flush<R, NF>(&a, sm, nq);
 }
 
 template <typename R, int NF, int MODE = 0>
@@ -613,26 +836,22 @@ __global__ void __launch_bounds__(256) near3d_batch(const EvalArgs *args, const 
 }
 
 // Batched near targets from the pairs' near lists (filled by a MODE-1
-// near3d_batch pass): every CTA walks the pairs in order, and within a pair the
-// list is spread over the grid starting at a CTA that rotates by the previous
-// pairs' block counts, so that small lists land on different CTAs.
+// near3d_batch pass): the pairs' tiles form one list, pair after pair, dealt out to the
+// warps of the grid in turn, so that the warps are in one or two pairs' grids
+// at a time and every warp has its share of the whole.
 template <typename R, int NF>
-__global__ void __launch_bounds__(256) near3d_list_batch(const EvalArgs *args, int np)
+__global__ void __launch_bounds__(32 * NEAR_WARPS) near3d_list_batch(const EvalArgs *args, int np)
 {
-    __shared__ EvalArgs sa;
-    int rot = 0;
+    __shared__ __align__(16) NearWarp<R, NF> smem[NEAR_WARPS];
+    NearWarp<R, NF> &sm = smem[threadIdx.x >> 5];
+    int t = blockIdx.x * NEAR_WARPS + (threadIdx.x >> 5), nq = 0;
     for (int p = 0; p < np; ++p) {
-        __syncthreads();
-        if (threadIdx.x == 0) sa = args[p];
-        __syncthreads();
-        const int nnear = sa.far_count[GF_NEAR_SLOT];
-        const int count = nnear + sa.far_count[GF_FGRID_SLOT];
-        const double ih1 = 1.0 / sa.h1, ih2 = 1.0 / sa.h2, ih3 = 1.0 / sa.h3;
-        const int cta = (int)((blockIdx.x + (unsigned)rot) % gridDim.x);
-        for (int j = cta * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x)
-            list_point<R, NF>(sa, j, nnear, ih1, ih2, ih3);
-        rot = (int)((rot + (count + blockDim.x - 1) / blockDim.x) % gridDim.x);
+        const int nnear = args[p].far_count[GF_NEAR_SLOT], nfg = args[p].far_count[GF_FGRID_SLOT];
+        const int tiles = ((nnear + 31) >> 5) + ((nfg + 31) >> 5);
+        for (; t < tiles; t += gridDim.x * NEAR_WARPS) near_list_tile<R, NF>(args, p, t, nnear, nfg, sm, nq);
+        t -= tiles;
     }
+    if (nq) sing_flush<R, NF>(args, sm, nq);
 }
 
 // ---------------------------------------------------------------------------
@@ -2519,6 +2738,14 @@ int resident_grid(int nsm)
     return per * nsm;
 }
 
+// The same for the near list: no more CTAs than the targets have tiles.
+template <void (*K)(const EvalArgs)>
+int near_grid(int64_t n, int nsm)
+{
+    const int64_t want = (n / 32 + 1) / NEAR_WARPS + 1;
+    return (int)std::min<int64_t>(want, resident_grid<K>(nsm));
+}
+
 // Concurrent far kernels of a Helmholtz double-precision plan: the double
 // kernel gives up FAR_F64_DROP of its resident CTAs per SM, and the float-tail
 // kernel (64-thread CTAs) fills the registers left free, so that both run at
@@ -2616,7 +2843,7 @@ cudaError_t launch_eval_t(const EvalArgs &a0, cudaStream_t s, cudaEvent_t ev_mid
         // with a near list: classify, then the near targets in full warps
         if (a.near_idx) {
             near3d<R, 1, 1><<<(int)blocks, 256, 0, s>>>(a);
-            near3d_list<R, 1><<<(int)blocks, 256, 0, s>>>(a);
+            near3d_list<R, 1><<<near_grid<near3d_list<R, 1>>(a.n, nsm), 32 * NEAR_WARPS, 0, s>>>(a);
         } else {
             near3d<R, 1><<<(int)blocks, 256, 0, s>>>(a);
         }
@@ -2634,7 +2861,7 @@ cudaError_t launch_eval_t(const EvalArgs &a0, cudaStream_t s, cudaEvent_t ev_mid
     } else {
         if (a.near_idx) {
             near3d<R, 7, 1><<<(int)blocks, 256, 0, s>>>(a);
-            near3d_list<R, 7><<<(int)blocks, 256, 0, s>>>(a);
+            near3d_list<R, 7><<<near_grid<near3d_list<R, 7>>(a.n, nsm), 32 * NEAR_WARPS, 0, s>>>(a);
         } else {
             near3d<R, 7><<<(int)blocks, 256, 0, s>>>(a);
         }
@@ -2654,35 +2881,29 @@ cudaError_t launch_eval_t(const EvalArgs &a0, cudaStream_t s, cudaEvent_t ev_mid
     return cudaGetLastError();
 }
 
+template <typename R, int NF>
+cudaError_t launch_eval_batch_nf(const EvalBatch &b, cudaStream_t s)
+{
+    // classification, then the near targets in full warps
+    int dev = 0, per = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, near3d_list_batch<R, NF>, 32 * NEAR_WARPS, 0) != cudaSuccess || per < 1) {
+        cudaGetLastError();
+        per = 1;
+    }
+    near3d_batch<R, NF, 1><<<b.grid_near, 256, 0, s>>>(b.args, b.prefix, b.np);
+    near3d_list_batch<R, NF><<<per * nsm, 32 * NEAR_WARPS, 0, s>>>(b.args, b.np);
+    far_scatter_batch<<<b.grid_scatter, 256, 0, s>>>(b.args, b.np, b.scatter_per_pair);
+    far3d_batch<R, NF><<<b.grid_far, b.block_far, 0, s>>>(b.args, b.np);
+    gf_count_launch(4);
+    return cudaGetLastError();
+}
+
 template <typename R>
 cudaError_t launch_eval_batch_t(const EvalBatch &b, cudaStream_t s)
 {
-    if (b.nf == 1) {
-        if (b.near_lists) {
-            // classification, then the near targets in full warps
-            int per = 0, dev = 0, nsm = 1;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, near3d_list_batch<R, 1>, 256, 0) != cudaSuccess ||
-                per < 1) {
-                cudaGetLastError();
-                per = 1;
-            }
-            near3d_batch<R, 1, 1><<<b.grid_near, 256, 0, s>>>(b.args, b.prefix, b.np);
-            near3d_list_batch<R, 1><<<per * nsm, 256, 0, s>>>(b.args, b.np);
-            gf_count_launch(1);
-        } else {
-            near3d_batch<R, 1><<<b.grid_near, 256, 0, s>>>(b.args, b.prefix, b.np);
-        }
-        far_scatter_batch<<<b.grid_scatter, 256, 0, s>>>(b.args, b.np, b.scatter_per_pair);
-        far3d_batch<R, 1><<<b.grid_far, b.block_far, 0, s>>>(b.args, b.np);
-    } else {
-        near3d_batch<R, 7><<<b.grid_near, 256, 0, s>>>(b.args, b.prefix, b.np);
-        far_scatter_batch<<<b.grid_scatter, 256, 0, s>>>(b.args, b.np, b.scatter_per_pair);
-        far3d_batch<R, 7><<<b.grid_far, b.block_far, 0, s>>>(b.args, b.np);
-    }
-    gf_count_launch(3);
-    return cudaGetLastError();
+    return b.nf == 1 ? launch_eval_batch_nf<R, 1>(b, s) : launch_eval_batch_nf<R, 7>(b, s);
 }
 
 }  // namespace

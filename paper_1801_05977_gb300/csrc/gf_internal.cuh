@@ -173,7 +173,18 @@ struct PropEntry {
     float c1f, c2f, brf, ibrf;
 };
 
+// Constants of the 3D gathers: stencil coordinates u - 1/2 = x ih + o of the near grid
+// and of the far-region grid, alpha/(2 pi), node spacings in float and the square
+// of the distance (a little above 2 eps) within which the singular part is formed.
+struct GatherArgs {
+    double ih1, o1, ih2, o2, ih3, o3;
+    double fih1, fo1, fihz, foz;
+    double al1, al2;
+    float h1, h2, rs2;
+};
+
 struct EvalArgs {
+    GatherArgs ga;
     int dim;
     int M1, M2, M3;
     int P1, P2, P3;
@@ -291,7 +302,6 @@ struct EvalBatch {
     int nf;
     int grid_near, grid_scatter, grid_far, block_far;
     int scatter_per_pair;
-    bool near_lists;        // per-pair near lists present (EvalArgs::near_idx): classify, then near3d_list_batch
 };
 
 // degree of the panels' interpolants; row length of SynthArgs::Ef

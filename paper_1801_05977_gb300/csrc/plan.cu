@@ -873,6 +873,23 @@ gf_status gf_plan_eval_args(gf_plan_t p, const double *dev_xyz, int64_t n, int w
         a.fhz = p->fhz;
         a.fzmax = p->fzmax;
         a.fh1 = a.fh2 = 2.0 * GF_PI / p->fM;
+        a.ga.fih1 = 1.0 / a.fh1;
+        a.ga.fo1 = 0.5 * p->fM - 0.5;
+        a.ga.fihz = 1.0 / a.fhz;
+        a.ga.foz = -a.fz0 * a.ga.fihz - 0.5;
+    }
+    if (p->dim == 3) {
+        a.ga.ih1 = 1.0 / a.h1;
+        a.ga.o1 = 0.5 * a.M1 - 0.5;
+        a.ga.ih2 = 1.0 / a.h2;
+        a.ga.o2 = 0.5 * a.M2 - 0.5;
+        a.ga.ih3 = 1.0 / a.h3;
+        a.ga.o3 = 0.5 * a.M3 - 0.5;
+        a.ga.al1 = a.a1 / (2.0 * GF_PI);
+        a.ga.al2 = a.a2 / (2.0 * GF_PI);
+        a.ga.h1 = (float)a.h1;
+        a.ga.h2 = (float)a.h2;
+        a.ga.rs2 = (float)((2.0 * a.eps + 2e-5) * (2.0 * a.eps + 2e-5) * (1.0 + 1e-5));
     }
     *a_out = a;
     return GF_OK;
