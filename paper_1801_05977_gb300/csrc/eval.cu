@@ -498,6 +498,10 @@ __device__ __forceinline__ void near_point(const EvalArgs &a, int64_t i, double 
 // is the limit, and 28 lanes of 32 and the shuffled sums would cost more of it.)
 // The targets next to a source wait in the warp's queue until a full warp of
 // them is there: most warps hold one or two, and would all pay for the singular part.
+// 600,000 near targets of a million (cold), one thread a target -> this: Helmholtz 128 x 128 x 64
+// float 228 -> 103 us, double 534 -> 349 us (170 of its 250 double operations a target are the
+// interpolation); Maxwell 256 x 256 x 64 float 802 -> 320 us; with 400,000 more in a 512 x 512 far grid
+// 290 -> 130 us; 64 batched pairs, 3.4 million near targets, 1345 -> 342 us.
 // ---------------------------------------------------------------------------
 constexpr int NEAR_WARPS = 4;
 template <typename R> constexpr int near_ws() { return sizeof(R) == 4 ? 20 : 22; }  // w23 [16], w1 [4] (and bank padding)
