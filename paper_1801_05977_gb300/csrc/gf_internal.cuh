@@ -339,7 +339,21 @@ cudaError_t gf_launch_synth_batch(const SynthBatch &b, int precision, cudaStream
 cudaError_t gf_launch_eval_batch(const EvalBatch &b, int precision, cudaStream_t s);
 cudaError_t gf_launch_series_tables(const EvalArgs &a, int precision, double2 *exptab, longlong2 *trig, PropEntry *prop, int *nprop,
                                     const int pbox[4], cudaStream_t s);
-cudaError_t gf_launch_e_table(const double *tt, int Q, int Mlast, double qs, double2 *E, float2 *Ef, cudaStream_t s);
+// panels.cu: the nodes' tables and, from their powers, the panels of the radial transforms
+struct NodeTables {
+    int Q, Mlast;
+    double qs;
+    const double *tt, *rr, *P0, *P1;
+    const double2 *B;
+    const double *rrd, *wyd;  // 2D derivative plans: 2 Q nodes of [0, 2 eps] and weights, else null
+    double2 *E;
+    float2 *Ef;
+    double2 *Bp;              // 3D: powers, or null
+    double *W;                // 2D: powers, or null
+};
+size_t gf_node_powers(int dim, int Q, bool deriv, double eps);
+cudaError_t gf_launch_node_tables(const NodeTables &a, cudaStream_t s);
+cudaError_t gf_launch_panels(const NodeTables &a, int dim, int npan, double2 *out, float2 *outf, double2 *dout, cudaStream_t s);
 // far-region grid: the planes' coefficients into a.work ([nf][L3count][M2][M1], FFT
 // order), then the x2 and x1 passes into a.grid (a.zlinear set)
 cudaError_t gf_launch_far_grid(const SynthArgs &a, int precision, double k, double a1, double a2, double z0,

@@ -405,7 +405,7 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     // Piecewise Chebyshev interpolants (degree 14, panels of width 2) of the
     // radial transforms on [0, s_max], s_max >= the largest frequency norm:
     // 3D h(s) = sum_m B_m sin(s r_m)/s, 2D the Bessel sums of F1-hat, F2-hat.
-    // (computed on the device from the quadrature tables, see gf_launch_cheb_table)
+    // (computed on the device from the quadrature tables, see panels.cu)
     const int hdeg = GF_HDEG;
     const double hpan = 2.0;
     int hnpan = 1;
@@ -445,7 +445,8 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     const size_t host_tab_bytes = sizeof(double) * Qa + sizeof(double2) * Q + (deriv ? sizeof(double) * 4 * Q : 0);
     const bool ftabs = dim == 3 && tr.precision == GF_FP32_SPLIT;  // float copies for the split plans' coefficients
     const size_t dcheb_n = deriv ? 3 * hcheb_n : 0;
-    const size_t tab_bytes = host_tab_bytes + sizeof(double2) * (E_n + hcheb_n + dcheb_n) +
+    const size_t npow = gf_node_powers(dim, Q, deriv, eps), npow2 = (npow + 1) / 2;
+    const size_t tab_bytes = host_tab_bytes + sizeof(double2) * (E_n + hcheb_n + dcheb_n + npow2) +
                              (ftabs ? sizeof(float2) * (E_n + hcheb_n) : 0);
     const size_t work_bytes = gf_plan_work_bytes(p);
     void *work = nullptr;
@@ -468,7 +469,8 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
         double2 *d_B = (double2 *)(d_tt + Qa);
         double *d_rrd = (double *)(d_B + Q), *d_wyd = d_rrd + (deriv ? 2 * Q : 0);
         double2 *d_E = (double2 *)(d_wyd + (deriv ? 2 * Q : 0)), *d_H = d_E + E_n, *d_D = d_H + hcheb_n;
-        float2 *d_Ef = ftabs ? (float2 *)(d_D + dcheb_n) : nullptr, *d_Hf = ftabs ? d_Ef + E_n : nullptr;
+        double2 *d_pow = d_D + dcheb_n;
+        float2 *d_Ef = ftabs ? (float2 *)(d_pow + npow2) : nullptr, *d_Hf = ftabs ? d_Ef + E_n : nullptr;
         {
             std::vector<char> pack(host_tab_bytes, 0);
             char *hb = pack.data();
@@ -482,10 +484,28 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
                 memcpy(hb + ((char *)d_rrd - tb), rrd.data(), sizeof(double) * 2 * Q);
                 memcpy(hb + ((char *)d_wyd - tb), wyd.data(), sizeof(double) * 2 * Q);
             }
-            if ((e = gf_stage_upload(tb, hb, host_tab_bytes, st)) != cudaSuccess ||
-                (e = gf_launch_e_table(d_tt, Q, Mlast, GF_PI / ct, d_E, d_Ef, st)) != cudaSuccess ||
-                (e = gf_launch_cheb_table(dim, d_rr, d_B, d_P0, d_P1, Q, hnpan, hdeg, hpan, d_H, d_Hf, st)) != cudaSuccess ||
-                (deriv && (e = gf_launch_cheb_deriv(d_rrd, d_wyd, 2 * Q, hnpan, hdeg, hpan, d_D, st)) != cudaSuccess)) {
+            NodeTables nt{};
+            nt.Q = Q;
+            nt.Mlast = Mlast;
+            nt.qs = GF_PI / ct;
+            nt.tt = d_tt;
+            nt.rr = d_rr;
+            nt.P0 = d_P0;
+            nt.P1 = d_P1;
+            nt.B = d_B;
+            nt.rrd = deriv ? d_rrd : nullptr;
+            nt.wyd = deriv ? d_wyd : nullptr;
+            nt.E = d_E;
+            nt.Ef = d_Ef;
+            nt.Bp = npow && dim == 3 ? d_pow : nullptr;
+            nt.W = npow && dim == 2 ? (double *)d_pow : nullptr;
+            if ((e = gf_stage_upload(tb, hb, host_tab_bytes, st)) == cudaSuccess && (e = gf_launch_node_tables(nt, st)) == cudaSuccess) {
+                if (npow)
+                    e = gf_launch_panels(nt, dim, hnpan, d_H, d_Hf, d_D, st);
+                else if ((e = gf_launch_cheb_table(dim, d_rr, d_B, d_P0, d_P1, Q, hnpan, hdeg, hpan, d_H, d_Hf, st)) == cudaSuccess && deriv)
+                    e = gf_launch_cheb_deriv(d_rrd, d_wyd, 2 * Q, hnpan, hdeg, hpan, d_D, st);
+            }
+            if (e != cudaSuccess) {
                 st_err = fail(GF_ERR_CUDA, "gf_plan: tables: %s", cudaGetErrorString(e));
                 break;
             }

@@ -835,7 +835,9 @@ void synth_config_t(SynthArgs &a, int tj_max, size_t sm[3])
                (a.deriv && a.k2 > 0.0 ? TJ * sizeof(double2) * (a.Q + 1) + 16 : 0);
     };
     int TJ = tj_max;
-    while (TJ > 1 && (TJ > ncols || bytes(TJ) > 160 * 1024)) TJ >>= 1;
+    // 2D: few columns, so few per CTA that there are CTAs for 152 SMs (64 x 64: 61 -> 31 us with 1 for 8;
+    // 256 x 256 derivatives 301 -> 158 us)
+    while (TJ > 1 && (TJ > ncols || bytes(TJ) > 160 * 1024 || (a.dim == 2 && ncols / TJ < 152))) TJ >>= 1;
     a.TJ = TJ;
     sm[0] = bytes(TJ);
     // 3D split plans have a first pass of their own (wider tiles: its columns are the lanes)
@@ -1138,23 +1140,6 @@ cudaError_t gf_launch_cheb_deriv(const double *rr, const double *wy, int Q2, int
     return cudaGetLastError();
 }
 
-// E[b][m] = e^{i q_b t_m}, q_b = j qs (qs = pi / c~) with j = b for b < Mlast/2, else
-// b - Mlast (the last-axis frequencies of Eq. (fck-coef)), t_m the Gauss nodes
-// of the X' integrals.
-__global__ void e_table_kernel(const double *tt, int Q, int Mlast, double qs, double2 *E, float2 *Ef)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Mlast * Q; i += gridDim.x * blockDim.x) {
-        const int b = i / Q, m = i - b * Q;
-        const int jl = b < Mlast / 2 ? b : b - Mlast;
-        const double q = (double)jl * qs;
-        double sv, cv;
-        sincos(q * tt[m], &sv, &cv);
-        E[i] = make_double2(cv, sv);
-        // float copy by node, [m][b] for b <= Mlast/2 (the coefficients formed)
-        if (Ef && b <= Mlast / 2) Ef[(size_t)m * GF_EF_ROW(Mlast) + b] = make_float2((float)cv, (float)sv);
-    }
-}
-
 namespace {
 // Far-region grid coefficients (the far branch's series (he) on planes): for
 // in-plane index n (FFT order b) and plane m at z = z0 + m hz,
@@ -1255,15 +1240,6 @@ cudaError_t gf_launch_far_grid(const SynthArgs &a, int precision, double k, doub
 {
     return precision == GF_FP64 ? launch_far_grid_t<double>(a, k, a1, a2, z0, hz, s)
                                 : launch_far_grid_t<float>(a, k, a1, a2, z0, hz, s);
-}
-
-cudaError_t gf_launch_e_table(const double *tt, int Q, int Mlast, double qs, double2 *E, float2 *Ef, cudaStream_t s)
-{
-    int blocks = (Mlast * Q + 255) / 256;
-    if (blocks > 1024) blocks = 1024;
-    e_table_kernel<<<blocks, 256, 0, s>>>(tt, Q, Mlast, qs, E, Ef);
-    gf_count_launch(1);
-    return cudaGetLastError();
 }
 
 cudaError_t gf_launch_cheb_table(int dim, const double *rr, const double2 *B, const double *P0, const double *P1, int Q,
