@@ -2621,109 +2621,270 @@ __global__ void far3d_batch(const EvalArgs *args, int np)
 }
 
 // ---------------------------------------------------------------------------
-// 2D far kernel: G = e^{i2pi alpha m} (i/4pi) sum_n beta_n^{-1} e^{i alpha_n t + i beta_n |x2|}
-// (terms and sums in double for both precisions).  One warp per target: lane l
-// takes n = na + l, na + l + 32, ... (phase e^{i alpha_n t} from a sincos and the
-// step e^{i 32 t}), and the lanes' sums are added by shuffles.
-// ---------------------------------------------------------------------------
-// Term n of (ei) without its factor i/(4pi): beta_n, E_n = e^{i alpha_n t + i beta_n
-// |x2|} (p = e^{i alpha_n t} given) and E_n / beta_n (beta_n = b or i b, so the
-// quotient is E/b or -i E/b).
-__device__ __forceinline__ void ei_term(double kk, double aa, double z, double2 p, double2 &beta, double2 &E,
-                                        double2 &term)
-{
-    if (aa <= kk) {
-        const double b = sqrt((kk - aa) * (kk + aa)), ib = 1.0 / b;
-        double sz, cz;
-        sincos(b * z, &sz, &cz);
-        beta = make_double2(b, 0.0);
-        E = cmul(make_double2(cz, sz), p);
-        term = make_double2(E.x * ib, E.y * ib);
-    } else {
-        const double b = sqrt((aa - kk) * (aa + kk)), ib = 1.0 / b;
-        beta = make_double2(0.0, b);
-        E = cscale(p, exp(-b * z));
-        term = make_double2(E.y * ib, -E.x * ib);
-    }
-}
-
-// 2D far branch (|x2| > c): (ei) summed by one warp per target, lanes over n.
+// 2D far branch (|x2| > c): G = e^{i2pi alpha m} (i/4pi) sum_n beta_n^{-1} e^{i alpha_n t + i beta_n |x2|}
+// (ei), terms and sums in double for both precisions.
 // GF_OUT_GRAD adds the term-by-term derivatives (i alpha_n/beta_n) E_n and
 // i sgn(x2) E_n; GF_OUT_HESSDIFF sums, over the indices of both wave numbers'
 // truncation sets, -alpha_n^2 (E_n/beta_n - E'_n/beta'_n), -alpha_n sgn (E_n - E'_n)
 // and -(beta_n E_n - beta'_n E'_n) (primes: k2).
 // OUT: the output kind (GF_OUT_G, GF_OUT_GRAD or GF_OUT_HESSDIFF), one kernel
 // instance each so that the plain G sum carries none of the others' registers.
+//
+// The double pipe bounds it.  A CTA keeps b_n = |beta_n|, 1/b_n and alpha_n of the index
+// range of |x2| = c in shared memory, and e^{-j/64}.  The
+// evanescent indices' weights are real, so their sums sum_n w_n v^n, v = e^{it}, go by Horner's rule
+// in v^4, four terms to a group; e^{-b|x2|} is the table's entry and a degree-6 polynomial.
+// About 15, 21 and 38 double operations a term for G, GRAD and HESSDIFF against 60,
+// 65 and 120 with a square root, a quotient, exp and a phase step in every term.  The
+// propagating indices are summed apart.  A target is shared by as many
+// lanes (1 .. 32, a run of indices each) as give an SM up to four warps; more would cost
+// more than they hide (two sines and the powers of v per lane).  A CTA orders its targets
+// by |x2|, so that the lanes of a warp have runs of about the same length.
+// 10,000 targets, G 111 -> 49 us; 100,000: GRAD 998 -> 256, HESSDIFF 1597 -> 455 us (without the
+// ordering and the even shares of the CTAs 479 and 861).
+// ---------------------------------------------------------------------------
+constexpr int F2_THR = 512;
+constexpr int F2_TAB = 1024;            // indices kept (the middle of the range)
+constexpr int F2_Y = 48;                // the exponential's table, y < F2_Y
+constexpr int F2_S = 64;                // steps per unit of y
+
+// (|beta_n|, 1/|beta_n|), the first negative for a propagating n.
+__device__ __forceinline__ double2 ei_beta(double kk, double c1)
+{
+    const double aa = fabs(c1), b = sqrt(fabs(aa - kk) * (aa + kk));
+    return make_double2(aa > kk ? b : -b, 1.0 / b);
+}
+
+// e^{-y}, y >= 0 (else of no use, but finite): y = j/64 + r, |r| <= 1/128, T[j] = e^{-j/64};
+// truncation r^7/5040 < 4e-19.
+__device__ __forceinline__ double exp_neg_tab(double y, const double *T)
+{
+    const double w = fma(y, (double)F2_S, 6755399441055744.0);
+    const int j = __double2loint(w);
+    if (y >= (double)F2_Y) return exp(-y);
+    const double r = fma(w - 6755399441055744.0, -1.0 / F2_S, y);
+    double p = fma(r, 1.0 / 720.0, -1.0 / 120.0);
+    p = fma(p, r, 1.0 / 24.0);
+    p = fma(p, r, -1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(p, r, -1.0);
+    const double t = T[max(j, 0)];
+    return fma(t, p * r, t);
+}
+
 template <typename R, int OUT>
-__global__ void __launch_bounds__(128) far2d(EvalArgs a)
+__global__ void __launch_bounds__(F2_THR) far2d(const __grid_constant__ EvalArgs a)
 {
     typedef typename cplx_t<R>::T C;
+    constexpr bool hess = OUT == GF_OUT_HESSDIFF, grad = OUT == GF_OUT_GRAD;
+    constexpr int ne = OUT == GF_OUT_G ? 1 : 3;
+    extern __shared__ double f2s[];
+    __shared__ double hi[F2_Y + 1], lo[F2_S];
+    __shared__ int bins[32], order[F2_THR];
+    double *T = f2s, *tc = T + F2_Y * F2_S + 1;
+    double2 *tb = reinterpret_cast<double2 *>(f2s + ((F2_Y * F2_S + 1 + F2_TAB + 1) & ~1)), *tb2 = tb + F2_TAB;
     C *out = reinterpret_cast<C *>(a.out);
     const int count = *a.far_count;
-    constexpr int ne = OUT == GF_OUT_G ? 1 : 3;
-    constexpr bool hess = OUT == GF_OUT_HESSDIFF, grad = OUT == GF_OUT_GRAD;
+    if (count == 0) return;
     const double kmax = (hess && a.k2 > a.k) ? a.k2 : a.k;
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int slot = gw; slot < count; slot += nw) {
-        const int idx = a.far_idx[slot];
+    // the kept indices: the range at |x2| = c, or its middle
+    const double Tc = a.T / a.c, Rc = sqrt(kmax * kmax + Tc * Tc);
+    const int mid = (int)rint(-a.a1), hw = (int)fmin(ceil(Rc) + 5.0, (double)(F2_TAB / 2));
+    const int tlo = mid - hw, tn = 2 * hw;
+    for (int i = threadIdx.x; i <= F2_Y; i += blockDim.x) hi[i] = exp(-(double)i);
+    for (int i = threadIdx.x; i < F2_S; i += blockDim.x) lo[i] = exp(-(double)i / F2_S);
+    for (int i = threadIdx.x; i < tn; i += blockDim.x) {
+        const double c1 = a.a1 + (tlo + i);
+        tc[i] = c1;
+        tb[i] = ei_beta(a.k, c1);
+        if (hess) tb2[i] = ei_beta(a.k2, c1);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= F2_Y * F2_S; i += blockDim.x) T[i] = hi[i / F2_S] * lo[i % F2_S];
+    __syncthreads();
+    // propagating indices: at most one past either end is not (skipped there)
+    int plo[2], phi[2];
+#pragma unroll
+    for (int q = 0; q < (hess ? 2 : 1); ++q) {
+        const double kk = q ? a.k2 : a.k;
+        plo[q] = (int)ceil(-a.a1 - kk - 1e-9 * kk);
+        phi[q] = (int)floor(-a.a1 + kk + 1e-9 * kk);
+    }
+    // the CTA's share of the targets; lanes per target
+    const int share = (count + gridDim.x - 1) / gridDim.x, c0 = blockIdx.x * share, c1e = min(count, c0 + share);
+    int lgl = 0;
+    while (lgl < 5 && (share << (lgl + 1)) <= 128) ++lgl;
+    const int lpt = 1 << lgl, sub = threadIdx.x & (lpt - 1), chunk = F2_THR >> lgl;
+    for (int base = c0; base < c1e; base += chunk) {
+        // order by the length of the sums, R ~ 1/|x2|: 32 bins
+        const int nt = min(chunk, c1e - base);
+        __syncthreads();
+        if (threadIdx.x < 32) bins[threadIdx.x] = 0;
+        __syncthreads();
+        int bin = 0, pos = 0, mine = 0;
+        if ((int)threadIdx.x < nt) {
+            mine = a.far_idx[base + threadIdx.x];
+            bin = min(31, (int)(32.f * (float)a.c / fabsf((float)a.x[2 * (size_t)mine + 1])));
+            pos = atomicAdd(&bins[bin], 1);
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const int v = bins[threadIdx.x];
+            int sum = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, sum, o);
+                if ((int)threadIdx.x >= o) sum += u;
+            }
+            bins[threadIdx.x] = sum - v;
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < nt) order[bins[bin] + pos] = mine;
+        __syncthreads();
+        const int slot = threadIdx.x >> lgl;
+        if (__ballot_sync(0xffffffffu, slot < nt) == 0u) continue;
+        const int idx = order[slot < nt ? slot : nt - 1];
         const double x1 = a.x[2 * (size_t)idx], x2 = a.x[2 * (size_t)idx + 1];
         double t, m;
         reduce_period(x1, t, m);
         const double z = fabs(x2), sg = x2 >= 0.0 ? 1.0 : -1.0;
         const double Tz = a.T * (1.0 / z);
-        const double R2 = kmax * kmax + Tz * Tz, Rr = sqrt(R2);
-        const int na = (int)floor(-a.a1 - Rr) - 1, nb = (int)ceil(-a.a1 + Rr) + 1;
-        double sp, cp, s32, c32;
-        sincos((a.a1 + (na + lane)) * t, &sp, &cp);
-        sincos(32.0 * t, &s32, &c32);
-        double2 p = make_double2(cp, sp);
-        const double2 step = make_double2(c32, s32);
+        const double Rr = sqrt(kmax * kmax + Tz * Tz);
+        const int na = (int)floor(-a.a1 - Rr), nb = (int)ceil(-a.a1 + Rr);
+        // runs of `per` indices outwards from mid, n = mid + k and n = mid - 1 - k: even lanes up, odd
+        // lanes down, one lane alone both; anchored at their inner ends, so that the
+        // large terms have small powers of v (groups of four: the outermost run may pass the
+        // truncation, which only adds accuracy)
+        const int lgr = lgl ? lgl - 1 : 0, kmx = max(nb - mid + 1, mid - na);
+        const int per = ((kmx + (1 << lgr) - 1) >> lgr) + 3 & ~3, k0 = (sub >> 1) * per;
+        double sv, cv;
+        sincos(t, &sv, &cv);
+        const double v2x = cv * cv - sv * sv, v2y = 2.0 * cv * sv;
+        const double v3x = v2x * cv - v2y * sv, v3y = v2x * sv + v2y * cv;
+        const double v4x = v2x * v2x - v2y * v2y, v4y = 2.0 * v2x * v2y;
         double acc[ne][2];
 #pragma unroll
         for (int e = 0; e < ne; ++e) acc[e][0] = acc[e][1] = 0.0;
-        for (int n = na + lane; n <= nb; n += 32, p = cmul(p, step)) {
-            const double c1 = a.a1 + n;
-            if (c1 * c1 > R2) continue;
-            const double aa = fabs(c1);
-            double2 beta, E, term;
-            ei_term(a.k, aa, z, p, beta, E, term);
-            if constexpr (!hess) {
-                acc[0][0] += term.x;
-                acc[0][1] += term.y;
-                if constexpr (grad) {
-                    acc[1][0] -= c1 * term.y;  // i c1 term
-                    acc[1][1] += c1 * term.x;
-                    acc[2][0] -= sg * E.y;     // i sgn E
-                    acc[2][1] += sg * E.x;
+        for (int q = 0; q < (lgl ? 1 : 2); ++q) {
+            const bool down = lgl ? sub & 1 : q;
+            const int n0 = down ? mid - 1 - k0 : mid + k0, d = down ? -1 : 1;
+            if (k0 >= kmx) continue;
+            const double dsv = down ? -sv : sv, w2y = down ? -v2y : v2y, w3y = down ? -v3y : v3y, w4y = down ? -v4y : v4y;
+            double h[ne][2];
+#pragma unroll
+            for (int e = 0; e < ne; ++e) h[e][0] = h[e][1] = 0.0;
+            for (int g = per - 4; g >= 0; g -= 4) {
+                double w[ne][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int n = n0 + d * (g + u), i = n - tlo;
+                    double c1;
+                    double2 q1, q2 = make_double2(0.0, 0.0);
+                    if ((unsigned)i < (unsigned)tn) {
+                        q1 = tb[i];
+                        c1 = ne > 1 ? tc[i] : 0.0;
+                        if (hess) q2 = tb2[i];
+                    } else {
+                        c1 = a.a1 + n;
+                        q1 = ei_beta(a.k, c1);
+                        if (hess) q2 = ei_beta(a.k2, c1);
+                    }
+                    // propagating indices weigh zero (the sign tested on the high word, off the double pipe)
+                    const double ex = exp_neg_tab(q1.x * z, T), e = __double2hiint(q1.x) > 0 ? ex : 0.0;
+                    if constexpr (!hess) {
+                        w[0][u] = e * q1.y;
+                        if constexpr (grad) {
+                            w[1][u] = c1 * w[0][u];
+                            w[2][u] = e;
+                        }
+                    } else {
+                        const double ex2 = exp_neg_tab(q2.x * z, T), e2 = __double2hiint(q2.x) > 0 ? ex2 : 0.0;
+                        w[0][u] = c1 * c1 * fma(e, q1.y, -(e2 * q2.y));
+                        w[1][u] = c1 * (e - e2);
+                        w[2][u] = fma(q1.x, e, -(q2.x * e2));
+                    }
                 }
-            } else {
-                double2 beta2, E2, term2;
-                ei_term(a.k2, aa, z, p, beta2, E2, term2);
-                const double2 d0 = csub(term, term2), d1 = csub(E, E2);
-                const double2 d2 = csub(cmul(beta, E), cmul(beta2, E2));
-                acc[0][0] -= c1 * c1 * d0.x;
-                acc[0][1] -= c1 * c1 * d0.y;
-                acc[1][0] -= c1 * sg * d1.x;
-                acc[1][1] -= c1 * sg * d1.y;
-                acc[2][0] -= d2.x;
-                acc[2][1] -= d2.y;
+#pragma unroll
+                for (int e = 0; e < ne; ++e) {
+                    const double x = fma(w[e][3], v3x, fma(w[e][2], v2x, fma(w[e][1], cv, w[e][0])));
+                    const double y = fma(w[e][3], w3y, fma(w[e][2], w2y, w[e][1] * dsv));
+                    const double nx = fma(h[e][0], v4x, fma(-h[e][1], w4y, x));
+                    h[e][1] = fma(h[e][0], w4y, fma(h[e][1], v4x, y));
+                    h[e][0] = nx;
+                }
+            }
+            // the run's phase e^{i alpha_{n0} t} and the factors of E_n = e^{-b|x2|} e^{i alpha_n t}, 1/beta_n = -i/b:
+            // G: -i; GRAD: 1, i sgn; HESSDIFF: i, -sgn, -i
+            double sp, cp;
+            sincos((a.a1 + n0) * t, &sp, &cp);
+#pragma unroll
+            for (int e = 0; e < ne; ++e) {
+                const double x = h[e][0] * cp - h[e][1] * sp, y = h[e][0] * sp + h[e][1] * cp;
+                if constexpr (!hess) {
+                    acc[e][0] += e == 0 ? y : e == 1 ? x : -sg * y;
+                    acc[e][1] += e == 0 ? -x : e == 1 ? y : sg * x;
+                } else {
+                    acc[e][0] += e == 0 ? -y : e == 1 ? -sg * x : y;
+                    acc[e][1] += e == 0 ? x : e == 1 ? -sg * y : -x;
+                }
             }
         }
+        // propagating indices of k (and, with the opposite sign, of k2)
 #pragma unroll
-        for (int e = 0; e < ne; ++e)
-            for (int o = 16; o > 0; o >>= 1) {
+        for (int q = 0; q < (hess ? 2 : 1); ++q) {
+            const double kk = q ? a.k2 : a.k, s = q ? -1.0 : 1.0;
+            for (int n = plo[q] + sub; n <= phi[q]; n += lpt) {
+                const double c1 = a.a1 + n;
+                const int i = n - tlo;
+                const double2 bq = (unsigned)i < (unsigned)tn ? (q ? tb2 : tb)[i] : ei_beta(kk, c1);
+                if (__double2hiint(bq.x) > 0) continue;
+                const double b = -bq.x, ib = bq.y;
+                double sz, cz;
+                sincos(fma(b, z, c1 * t), &sz, &cz);
+                if constexpr (!hess) {
+                    acc[0][0] = fma(cz, ib, acc[0][0]);
+                    acc[0][1] = fma(sz, ib, acc[0][1]);
+                    if constexpr (grad) {
+                        const double ci = c1 * ib;
+                        acc[1][0] = fma(-ci, sz, acc[1][0]);
+                        acc[1][1] = fma(ci, cz, acc[1][1]);
+                        acc[2][0] = fma(-sg, sz, acc[2][0]);
+                        acc[2][1] = fma(sg, cz, acc[2][1]);
+                    }
+                } else {
+                    const double f0 = -s * c1 * c1 * ib, f1 = -s * c1 * sg, f2 = -s * b;
+                    acc[0][0] = fma(f0, cz, acc[0][0]);
+                    acc[0][1] = fma(f0, sz, acc[0][1]);
+                    acc[1][0] = fma(f1, cz, acc[1][0]);
+                    acc[1][1] = fma(f1, sz, acc[1][1]);
+                    acc[2][0] = fma(f2, cz, acc[2][0]);
+                    acc[2][1] = fma(f2, sz, acc[2][1]);
+                }
+            }
+        }
+        for (int o = 1; o < lpt; o <<= 1)
+#pragma unroll
+            for (int e = 0; e < ne; ++e) {
                 acc[e][0] += __shfl_xor_sync(0xffffffffu, acc[e][0], o);
                 acc[e][1] += __shfl_xor_sync(0xffffffffu, acc[e][1], o);
             }
-        if (lane == 0) {
+        if (sub == 0 && slot < count) {
             const double2 lat = lattice_phase(a.a1, m, 0.0, 0.0);
             const double2 pre = cmul(lat, make_double2(0.0, 0.25 / GF_PI));
             for (int e = 0; e < ne; ++e)
                 store_out(out + (size_t)idx * ne + e, cmul(pre, make_double2(acc[e][0], acc[e][1])));
         }
     }
+}
+
+template <typename R, int OUT>
+cudaError_t launch_far2d(const EvalArgs &a, int nsm, cudaStream_t s)
+{
+    const size_t sm = sizeof(double) * ((F2_Y * F2_S + 1 + F2_TAB + 1) & ~1) + sizeof(double2) * F2_TAB * (OUT == GF_OUT_HESSDIFF ? 2 : 1);
+    cudaError_t e = cudaFuncSetAttribute(far2d<R, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    far2d<R, OUT><<<nsm, F2_THR, sm, s>>>(a);
+    return cudaSuccess;
 }
 
 // Persistent far grid: as many 128-thread CTAs as are resident at once (a
@@ -2837,12 +2998,10 @@ cudaError_t launch_eval_t(const EvalArgs &a0, cudaStream_t s, cudaEvent_t ev_mid
         else
             near2d<R, 6><<<(int)blocks, 256, 0, s>>>(a);
         if (ev_mid) cudaEventRecord(ev_mid, s);
-        if (a.which == GF_OUT_GRAD)
-            far2d<R, GF_OUT_GRAD><<<resident_grid<far2d<R, GF_OUT_GRAD>>(nsm), 128, 0, s>>>(a);
-        else if (a.which == GF_OUT_HESSDIFF)
-            far2d<R, GF_OUT_HESSDIFF><<<resident_grid<far2d<R, GF_OUT_HESSDIFF>>(nsm), 128, 0, s>>>(a);
-        else
-            far2d<R, GF_OUT_G><<<resident_grid<far2d<R, GF_OUT_G>>(nsm), 128, 0, s>>>(a);
+        cudaError_t e = a.which == GF_OUT_GRAD       ? launch_far2d<R, GF_OUT_GRAD>(a, nsm, s)
+                        : a.which == GF_OUT_HESSDIFF ? launch_far2d<R, GF_OUT_HESSDIFF>(a, nsm, s)
+                                                     : launch_far2d<R, GF_OUT_G>(a, nsm, s);
+        if (e != cudaSuccess) return e;
     } else if (a.nf == 1) {
         // with a near list: classify, then the near targets in full warps
         if (a.near_idx) {
