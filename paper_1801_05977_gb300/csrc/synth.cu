@@ -9,13 +9,10 @@
 // node index l standing for x = l h (mod period).  Each pass is a radix-2
 // Stockham autosort transform held in shared memory (one CTA owns a batch of
 // whole lines, so every pass reads and writes global memory exactly once).
-#include <cuda.h>
-#include <cudaTypedefs.h>
 #include <stdint.h>
 
-#include <mutex>
-
 #include "gf_internal.cuh"
+#include "synth_fft.cuh"
 #include "umma_gemm.cuh"
 
 namespace {
@@ -157,54 +154,6 @@ __device__ void stockham_inverse_grouped(C *x, C *y, int n, int lg, int nlines, 
 
 // tw[i] = e^{2 pi i i/n}, i < n/2, in the pass's precision (float passes take
 // the float sincospi: within an ulp, and no double arithmetic in a float pass)
-// The same transform on an interleaved tile: element j of line L at x[j NL + L]
-// (NL = 2^lgNL lines), the layout a 2D tensor copy of NL adjacent columns gives.
-// Consecutive threads take consecutive lines, so shared-memory accesses stay
-// contiguous.  Returns the buffer holding the result.
-template <typename C>
-__device__ C *stockham_inverse_il(C *x, C *y, int n, int lg, int lgNL, const C *tw)
-{
-    const int half = n >> 1, NL = 1 << lgNL;
-    int Ns = 1, lns = 0;
-    if (lg & 1) {
-        const int total = NL * half;
-        for (int it = threadIdx.x; it < total; it += blockDim.x) {
-            const int L = it & (NL - 1), j = it >> lgNL;
-            const C v0 = x[j * NL + L], v1 = x[(j + half) * NL + L];
-            y[(2 * j) * NL + L] = cadd(v0, v1);
-            y[(2 * j + 1) * NL + L] = csub(v0, v1);
-        }
-        __syncthreads();
-        C *t = x;
-        x = y;
-        y = t;
-        Ns = 2;
-        lns = 1;
-    }
-    const int q = n >> 2;
-    for (; Ns < n; Ns <<= 2, lns += 2) {
-        const int total = NL * q, sh = lg - 2 - lns;
-        for (int it = threadIdx.x; it < total; it += blockDim.x) {
-            const int L = it & (NL - 1), j = it >> lgNL, k = j & (Ns - 1);
-            const C a = x[j * NL + L];
-            const C b = cmul(x[(j + q) * NL + L], twiddle(tw, k << sh, half));
-            const C c = cmul(x[(j + 2 * q) * NL + L], twiddle(tw, (2 * k) << sh, half));
-            const C d = cmul(x[(j + 3 * q) * NL + L], twiddle(tw, (3 * k) << sh, half));
-            const C apc = cadd(a, c), amc = csub(a, c), bpd = cadd(b, d), bmd = csub(b, d);
-            const int o = ((j - k) << 2) + k;
-            y[o * NL + L] = cadd(apc, bpd);
-            y[(o + Ns) * NL + L] = cmk(amc.x - bmd.y, amc.y + bmd.x);
-            y[(o + 2 * Ns) * NL + L] = csub(apc, bpd);
-            y[(o + 3 * Ns) * NL + L] = cmk(amc.x + bmd.y, amc.y - bmd.x);
-        }
-        __syncthreads();
-        C *t = x;
-        x = y;
-        y = t;
-    }
-    return x;
-}
-
 template <typename R>
 __device__ void load_twiddles(typename cplx_t<R>::T *tw, int n)
 {
@@ -494,31 +443,29 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
 }
 
 // Middle pass (3D only): inverse transform along x2 for fixed (field, x3 node, b1-tile);
-// only the x3 nodes of the stored planes are transformed.
+// only the x3 nodes of the stored planes are transformed.  The first stage reads and the
+// last one writes the work buffer itself (64 bytes a row and field in float): as fast as tensor-map
+// copies of the tile into and out of shared memory (128 x 128 x 37 double 28 us either way, float
+// 5.6), and batched, 64 pairs, 551 -> 249 us against a staged tile of strided lines.
 template <typename R>
 __device__ void synth_x2_body(const SynthArgs &a, int bx, int y, int f, unsigned char *smem)
 {
     typedef typename cplx_t<R>::T C;
     const int n = a.M2, TJ = a.TJ2, lg2 = a.lg2;
-    // x3 node a3first + y, stored at plane y of the (compact) work buffer
+    // x3 node a3first + y, stored at plane y of the (compact) work buffer; the CTA owns its columns,
+    // so the last stage writes where the first one read
+    const int lgT = 31 - __clz(TJ);
     C *tw = reinterpret_cast<C *>(smem);
     C *buf0 = tw + (n >> 1);
     C *buf1 = buf0 + TJ * n;
-    const int b10 = bx * TJ;
     // work plane L3count (half-grid Maxwell plans) holds the Nyquist row of the odd fields only
     if (y == a.L3count && f != 4 && f != 5) return;
-    C *W = reinterpret_cast<C *>(a.work) + ((size_t)f * (a.L3count + a.nyq) + y) * (size_t)a.M2 * a.M1;
+    C *W = reinterpret_cast<C *>(a.work) + ((size_t)f * (a.L3count + a.nyq) + y) * (size_t)a.M2 * a.M1 + bx * TJ;
+    const int M1 = a.M1;
     load_twiddles<R>(tw, n);
-    for (int i = threadIdx.x; i < TJ * n; i += blockDim.x) {
-        int t = i % TJ, b2 = i / TJ;
-        buf0[t * n + b2] = W[(size_t)b2 * a.M1 + b10 + t];
-    }
-    __syncthreads();
-    C *res = stockham_inverse(buf0, buf1, n, lg2, TJ, tw);
-    for (int i = threadIdx.x; i < TJ * n; i += blockDim.x) {
-        int t = i % TJ, l2 = i / TJ;
-        W[(size_t)l2 * a.M1 + b10 + t] = res[t * n + l2];
-    }
+    fft_cols(
+        buf0, buf1, n, lg2, lgT, tw, [&](int b2, int t) { return W[(size_t)b2 * M1 + t]; },
+        [&](int l2, int t, C v) { W[(size_t)l2 * M1 + t] = v; });
 }
 
 __device__ __forceinline__ int pad_dests(int a_node, int M, int *p)
@@ -531,7 +478,8 @@ __device__ __forceinline__ int pad_dests(int a_node, int M, int *p)
     return nd;
 }
 
-// Last pass: inverse transform along x1 of RB1 consecutive rows (all fields),
+// Last pass (one field: the last stage writes the grid's rows itself; 128 x 128 x 37 float 12 -> 6 us,
+// batched 690 -> 271 us): inverse transform along x1 of RB1 consecutive rows (all fields),
 // then scatter into the padded, field-interleaved gather grid G[p3][p2][p1][f],
 // where padded index p = a + 1 holds node a = (l + M/2) mod M, i.e. x = -pi + a h
 // (x3: -c~ + a h3), with one halo node before and two after on every periodic
@@ -570,9 +518,41 @@ __device__ void synth_x1_body(const SynthArgs &a, int blk, unsigned char *smem, 
         umma::mbar_wait_n(umma::smem_u32(bar), parity, umma::WAIT_LIMIT);
     }
     __syncthreads();
+    C *G = reinterpret_cast<C *>(a.grid);
+    if (nf == 1) {
+        // one field: the last stage writes the padded rows.  A row's copies in the grid (halo
+        // rows and planes): their offsets, by one thread a row
+        __shared__ int ndst[8];
+        __shared__ int64_t dst[8][9];
+        if (threadIdx.x < RB) {
+            const int row = row0 + threadIdx.x, lgm = 31 - __clz(a.M2);
+            const int y = a.dim == 3 ? row >> lgm : 0, l2 = row & (a.M2 - 1);
+            int p2[3], p3[3] = {a.zlinear ? a.a3first + y : 0, 0, 0}, nd = 0;
+            const int n2 = pad_dests((l2 + (a.M2 >> 1)) & (a.M2 - 1), a.M2, p2);
+            const int n3 = a.dim == 3 && !a.zlinear ? pad_dests(a.a3first + y, a.M3, p3) : 1;
+            for (int d3 = 0; d3 < n3; ++d3) {
+                const int q3 = p3[d3] - a.Q3lo;
+                if (q3 < 0 || q3 >= a.P3) continue;  // only the stored planes Q3lo .. Q3lo + P3 - 1
+                for (int d2 = 0; d2 < n2; ++d2) dst[threadIdx.x][nd++] = ((int64_t)q3 * a.P2 + p2[d2]) * a.P1;
+            }
+            ndst[threadIdx.x] = nd;
+        }
+        // (the first stage's barrier orders this before the last stage)
+        fft_rows(
+            buf1, buf0, n, lg1, RB, tw, [&](int b, int t) { return buf0[t * n + b]; },
+            [&](int l, int t, C v) {
+                const int p1 = ((l + (n >> 1)) & (n - 1)) + 1;
+                for (int d = 0; d < ndst[t]; ++d) {
+                    C *g = G + dst[t][d];
+                    g[p1] = v;
+                    if (p1 <= 2) g[p1 + n] = v;
+                    if (p1 == n) g[0] = v;
+                }
+            });
+        return;
+    }
     stockham_inverse_grouped(buf0, buf1, n, lg1, RB * nf, RB, tw);
     const C *res = buf0;
-    C *G = reinterpret_cast<C *>(a.grid);
     const int rowlen = a.P1 * nf;
     for (int r = 0; r < RB; ++r) {
         const int row = row0 + r;
@@ -596,8 +576,7 @@ __device__ void synth_x1_body(const SynthArgs &a, int blk, unsigned char *smem, 
                 C *dst = NG + (size_t)p2[d2] * a.P1 * 2;
                 for (int i = threadIdx.x; i < 2 * a.P1; i += blockDim.x) {
                     const int p1 = i >> 1, f = 4 + (i & 1);
-                    const int a1 = (p1 - 1 + n) % n;
-                    dst[i] = rr[f * fs + (a1 + (n >> 1)) % n];
+                    dst[i] = rr[f * fs + ((p1 - 1 + (n >> 1)) & (n - 1))];
                 }
             }
             continue;
@@ -617,10 +596,8 @@ __device__ void synth_x1_body(const SynthArgs &a, int blk, unsigned char *smem, 
             for (int d2 = 0; d2 < n2; ++d2) {
                 C *dst = G + ((size_t)q3 * a.P2 + p2[d2]) * rowlen;
                 for (int i = threadIdx.x; i < rowlen; i += blockDim.x) {
-                    int p1 = i / nf, f = i - p1 * nf;
-                    int a1 = (p1 - 1 + n) % n;
-                    int l1 = (a1 + (n >> 1)) % n;
-                    dst[i] = rr[f * fs + l1];
+                    const int p1 = i / nf, f = i - p1 * nf;
+                    dst[i] = rr[f * fs + ((p1 - 1 + (n >> 1)) & (n - 1))];
                 }
             }
         }
@@ -652,65 +629,6 @@ __device__ __forceinline__ void init_copy_barrier(uint64_t *bar)
     __syncthreads();
 }
 
-// Middle pass with tensor-map copies (single plans): the TJ columns b10 .. b10+TJ-1
-// of the M2 rows of plane (f, y) are one 2D box of the work buffer seen as a
-// [rows][M1] matrix of 8-byte units (a complex is U = sizeof(C)/8 units), loaded
-// by cp.async.bulk.tensor in boxes of at most 256 rows into an interleaved tile
-// [b2][t], transformed there, and written back the same way by a TMA store.
-// The box's first unit x = b10 U is even (TJ >= 2), so x * 8 bytes is a multiple
-// of 16 as the tensor copy requires.
-constexpr int X2_BOX_ROWS = 256;
-
-template <typename R>
-__global__ void __launch_bounds__(256) synth_x2_pass_tma(SynthArgs a, const __grid_constant__ CUtensorMap tm)
-{
-    typedef typename cplx_t<R>::T C;
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bar;
-    const int n = a.M2, TJ = a.TJ2, lg2 = a.lg2;
-    const int bx = blockIdx.x, y = blockIdx.y, f = blockIdx.z;
-    if (y == a.L3count && f != 4 && f != 5) return;  // the Nyquist plane is only for xz, yz
-    int lgTJ = 0;
-    while ((1 << lgTJ) < TJ) ++lgTJ;
-    C *tw = reinterpret_cast<C *>(smem);
-    C *buf0 = reinterpret_cast<C *>(smem + ((sizeof(C) * (n >> 1) + 127) & ~(size_t)127));
-    C *buf1 = buf0 + TJ * n;
-    const int U = (int)(sizeof(C) / 8);
-    const int x0 = bx * TJ * U, row0 = (f * (a.L3count + a.nyq) + y) * n;
-    const int boxr = n < X2_BOX_ROWS ? n : X2_BOX_ROWS;
-    const uint64_t tmap = reinterpret_cast<uint64_t>(&tm);
-    init_copy_barrier(&bar);
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(umma::smem_u32(&bar)),
-                     "r"((uint32_t)(n * TJ * sizeof(C)))
-                     : "memory");
-        for (int r = 0; r < n; r += boxr)
-            asm volatile(
-                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-                    umma::smem_u32(buf0 + (size_t)r * TJ)),
-                "l"(tmap), "r"(x0), "r"(row0 + r), "r"(umma::smem_u32(&bar))
-                : "memory");
-    }
-    load_twiddles<R>(tw, n);
-    if (!umma::mbar_wait_n(umma::smem_u32(&bar), 0u, umma::WAIT_LIMIT)) {
-        if (a.err) atomicExch(a.err, 1);
-        umma::mbar_wait_n(umma::smem_u32(&bar), 0u, umma::WAIT_LIMIT);
-    }
-    __syncthreads();
-    C *res = stockham_inverse_il(buf0, buf1, n, lg2, lgTJ, tw);
-    // the transformed tile is read by the async proxy: order the generic writes first
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int r = 0; r < n; r += boxr)
-            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tmap),
-                         "r"(x0), "r"(row0 + r), "r"(umma::smem_u32(res + (size_t)r * TJ))
-                         : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-    }
-}
-
 template <typename R>
 __global__ void __launch_bounds__(256) synth_x1_pass(SynthArgs a)
 {
@@ -734,6 +652,19 @@ __device__ __forceinline__ int batch_pair(const int *prefix, int np, int vb)
     return lo;
 }
 
+// The pair of virtual block vb and, when it is not the one before, its arguments.
+__device__ __forceinline__ int batch_args(SynthArgs &sa, const SynthArgs *args, const int *prefix, int np, int vb, int &cur)
+{
+    if (cur < 0 || vb >= prefix[cur + 1]) {
+        cur = batch_pair(prefix, np, vb);
+        const int *src = reinterpret_cast<const int *>(args + cur);
+        for (int i = threadIdx.x; i < (int)(sizeof(SynthArgs) / sizeof(int)); i += blockDim.x)
+            reinterpret_cast<int *>(&sa)[i] = src[i];
+        __syncthreads();
+    }
+    return cur;
+}
+
 // Batched synthesis passes: one persistent launch per pass walks the
 // (pair, block) work list of all plans of a sweep; prefix[p] is the first
 // virtual block of pair p (prefix[np] = total).
@@ -743,10 +674,9 @@ __global__ void __launch_bounds__(256) synth_first_pass_batch(const SynthArgs *a
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ SynthArgs sa;
     const int total = prefix[np];
+    int cur = -1;
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const int p = batch_pair(prefix, np, vb);
-        if (threadIdx.x == 0) sa = args[p];
-        __syncthreads();
+        const int p = batch_args(sa, args, prefix, np, vb, cur);
         synth_first_pass_body<R, false>(sa, vb - prefix[p], smem);
         __syncthreads();
     }
@@ -758,10 +688,9 @@ __global__ void __launch_bounds__(256) synth_x2_pass_batch(const SynthArgs *args
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ SynthArgs sa;
     const int total = prefix[np];
+    int cur = -1;
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const int p = batch_pair(prefix, np, vb);
-        if (threadIdx.x == 0) sa = args[p];
-        __syncthreads();
+        const int p = batch_args(sa, args, prefix, np, vb, cur);
         int loc = vb - prefix[p];
         const int nbx = sa.M1 / sa.TJ2;
         const int bx = loc % nbx;
@@ -782,10 +711,9 @@ __global__ void __launch_bounds__(256) synth_x1_pass_batch(const SynthArgs *args
     init_copy_barrier(&bar);
     const int total = prefix[np];
     uint32_t phase = 0;
+    int cur = -1;
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x, phase ^= 1u) {
-        const int p = batch_pair(prefix, np, vb);
-        if (threadIdx.x == 0) sa = args[p];
-        __syncthreads();
+        const int p = batch_args(sa, args, prefix, np, vb, cur);
         synth_x1_body<R>(sa, vb - prefix[p], smem, &bar, phase);
         __syncthreads();
     }
@@ -858,53 +786,12 @@ void synth_config_t(SynthArgs &a, int tj_max, size_t sm[3])
     sm[2] = sizeof(C) * (a.M1 / 2 + (a.nf + 1) * RB1 * a.M1);
 }
 
-// cuTensorMapEncodeTiled from the driver (through the runtime's entry-point
-// query, so the library needs no link to libcuda); null when unavailable.
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
-{
-    static std::once_flag once;
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
-// Middle pass of a single plan: tensor-map copies when the tile allows them
-// (TJ >= 2 columns, a map the driver accepts), the plain staged loop otherwise.
 template <typename R>
-cudaError_t launch_x2(const SynthArgs &a, size_t smem_plain, cudaStream_t s)
+cudaError_t launch_x2(const SynthArgs &a, size_t smem, cudaStream_t s)
 {
-    typedef typename cplx_t<R>::T C;
-    const dim3 grid(a.M1 / a.TJ2, a.L3count + a.nyq, a.nf);
-    PFN_cuTensorMapEncodeTiled_v12000 enc = a.TJ2 >= 2 ? tensor_map_encoder() : nullptr;
-    if (enc) {
-        const int U = (int)(sizeof(C) / 8);
-        const cuuint64_t dims[2] = {(cuuint64_t)a.M1 * U, (cuuint64_t)a.M2 * (a.L3count + a.nyq) * a.nf};
-        const cuuint64_t strides[1] = {(cuuint64_t)a.M1 * sizeof(C)};
-        const cuuint32_t box[2] = {(cuuint32_t)(a.TJ2 * U), (cuuint32_t)(a.M2 < X2_BOX_ROWS ? a.M2 : X2_BOX_ROWS)};
-        const cuuint32_t estr[2] = {1, 1};
-        CUtensorMap tm;
-        if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, a.work, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
-            const size_t sm = ((sizeof(C) * (a.M2 >> 1) + 127) & ~(size_t)127) + 2 * sizeof(C) * a.TJ2 * a.M2;
-            cudaError_t e = cudaFuncSetAttribute(synth_x2_pass_tma<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-            synth_x2_pass_tma<R><<<grid, 256, sm, s>>>(a, tm);
-            gf_count_launch(1);
-            return cudaGetLastError();
-        }
-    }
-    cudaError_t e = cudaFuncSetAttribute(synth_x2_pass<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plain);
+    cudaError_t e = cudaFuncSetAttribute(synth_x2_pass<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    synth_x2_pass<R><<<grid, 256, smem_plain, s>>>(a);
+    synth_x2_pass<R><<<dim3(a.M1 / a.TJ2, a.L3count + a.nyq, a.nf), 256, smem, s>>>(a);
     gf_count_launch(1);
     return cudaGetLastError();
 }

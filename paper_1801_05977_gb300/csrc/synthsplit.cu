@@ -15,14 +15,15 @@
 // each) against sixteen FMAs.
 //
 // What bounds it: issue (the X' sums, 15 multiply-adds on a table entry each for h(s), the
-// transforms), about a third of the slots used; the store is 0.3 GB of the 1.5 ms below.
+// transforms), about a third of the slots used; the store is 0.3 GB of the 1.1 ms below.
 // Before, a CTA held 8 columns by [column][b]: half its threads had no item, each lane read its
 // own line of E, the double set-up ran on 8 lanes of a warp and the double columns held
-// their CTA up.  Batched, 64 pairs with 0.5 <= k <= 5 on 32^2 x 64 to 256^2 x 64: 5.86 -> 1.47 ms.
+// their CTA up.  Batched, 64 pairs with 0.5 <= k <= 5 on 32^2 x 64 to 256^2 x 64: 5.86 -> 1.14 ms.
 // One plan (cold): 128 x 128 x 64 85 -> 32 us, Maxwell 256 x 256 x 64 319 -> 125 us.
 #include <stdint.h>
 
 #include "gf_internal.cuh"
+#include "synth_fft.cuh"
 
 namespace {
 
@@ -79,90 +80,12 @@ __host__ __device__ inline UnitLay unit_lay(int n, int Q)
     return l;
 }
 
-__device__ __forceinline__ float2 cmulf(float2 a, float2 b)
-{
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ float2 addf(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 subf(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-
 __device__ void load_tw(float2 *tw, int n)
 {
     for (int i = threadIdx.x; i < (n >> 1); i += blockDim.x) {
         float s, c;
         sincospif(2.0f * (float)i / (float)n, &s, &c);
         tw[i] = make_float2(c, s);
-    }
-}
-
-// Inverse transforms (+ sign, unnormalised) of T = 2^lgT lines of n = 2^lg >= 8, Stockham
-// radix 4 after one radix-2 stage when lg is odd: element j of line t comes
-// from ld(j, t), output l goes to st(l, t, v), the stages between go through x
-// and y ([n][T] each).  The first stage reads and the last one writes without
-// a pass of their own.
-template <class Ld, class St>
-__device__ __forceinline__ void fft_lines(float2 *x, float2 *y, int n, int lg, int lgT, const float2 *tw, Ld ld, St st)
-{
-    const int half = n >> 1, q = n >> 2, T = 1 << lgT;
-    int Ns, lns;
-    if (lg & 1) {
-        for (int it = threadIdx.x; it < half << lgT; it += blockDim.x) {
-            const int t = it & (T - 1), j = it >> lgT;
-            const float2 v0 = ld(j, t), v1 = ld(j + half, t);
-            x[(2 * j) * T + t] = addf(v0, v1);
-            x[(2 * j + 1) * T + t] = subf(v0, v1);
-        }
-        Ns = 2;
-        lns = 1;
-    } else {
-        for (int it = threadIdx.x; it < q << lgT; it += blockDim.x) {
-            const int t = it & (T - 1), j = it >> lgT;
-            const float2 a = ld(j, t), b = ld(j + q, t), c = ld(j + 2 * q, t), d = ld(j + 3 * q, t);
-            const float2 apc = addf(a, c), amc = subf(a, c), bpd = addf(b, d), bmd = subf(b, d);
-            float2 *o = x + (4 * j) * T + t;
-            o[0] = addf(apc, bpd);
-            o[T] = make_float2(amc.x - bmd.y, amc.y + bmd.x);
-            o[2 * T] = subf(apc, bpd);
-            o[3 * T] = make_float2(amc.x + bmd.y, amc.y - bmd.x);
-        }
-        Ns = 4;
-        lns = 2;
-    }
-    __syncthreads();
-    auto tws = [&](int m) {
-        const float2 v = tw[m & (half - 1)];
-        return m < half ? v : make_float2(-v.x, -v.y);
-    };
-    for (;; Ns <<= 2, lns += 2) {
-        const bool last = Ns == q;
-        const int sh = lg - 2 - lns;
-        for (int it = threadIdx.x; it < q << lgT; it += blockDim.x) {
-            const int t = it & (T - 1), j = it >> lgT, k = j & (Ns - 1);
-            const float2 a = x[j * T + t];
-            const float2 b = cmulf(x[(j + q) * T + t], tw[k << sh]);
-            const float2 c = cmulf(x[(j + 2 * q) * T + t], tw[(2 * k) << sh]);
-            const float2 d = cmulf(x[(j + 3 * q) * T + t], tws((3 * k) << sh));
-            const float2 apc = addf(a, c), amc = subf(a, c), bpd = addf(b, d), bmd = subf(b, d);
-            const float2 o0 = addf(apc, bpd), o1 = make_float2(amc.x - bmd.y, amc.y + bmd.x), o2 = subf(apc, bpd),
-                         o3 = make_float2(amc.x + bmd.y, amc.y - bmd.x);
-            const int o = ((j - k) << 2) + k;
-            if (last) {
-                st(o, t, o0);
-                st(o + Ns, t, o1);
-                st(o + 2 * Ns, t, o2);
-                st(o + 3 * Ns, t, o3);
-            } else {
-                y[o * T + t] = o0;
-                y[(o + Ns) * T + t] = o1;
-                y[(o + 2 * Ns) * T + t] = o2;
-                y[(o + 3 * Ns) * T + t] = o3;
-            }
-        }
-        __syncthreads();
-        if (last) return;
-        float2 *z = x;
-        x = y;
-        y = z;
     }
 }
 
@@ -334,7 +257,7 @@ __device__ void tile_body(const SynthArgs &a, int blk, unsigned char *smem)
         // only the x3 nodes the last two passes transform (a3first .. a3first +
         // L3count - 1), compact: work plane y holds node a3first + y, whose output
         // index is l = (a3first + y + n/2) mod n
-        fft_lines(X, Y, n, lg, lgT, tw, ld, [&](int l, int, float2 v) {
+        fft_cols(X, Y, n, lg, lgT, tw, ld, [&](int l, int, float2 v) {
             const int y = (l - half - a.a3first) & (n - 1);
             if (y < a.L3count && mine) Wf[(size_t)y * ncols] = v;
         });
@@ -442,7 +365,7 @@ __device__ void unit_body(const SynthArgs &a, int u, unsigned char *smem)
             const float2 v = base[b <= half ? b : n - b];
             return odd && b > half ? make_float2(-v.x, -v.y) : v;
         };
-        fft_lines(X, Y, n, lg, 0, tw, ld, [&](int l, int, float2 v) {
+        fft_rows(X, Y, n, lg, 1, tw, ld, [&](int l, int, float2 v) {
             const int y = (l - half - a.a3first) & (n - 1);
             if (y < a.L3count) Wf[(size_t)y * ncols] = v;
         });
@@ -458,13 +381,13 @@ __device__ __forceinline__ void first_split_body(const SynthArgs &a, int blk, un
         tile_body(a, blk - a.ndbl, smem);
 }
 
-__global__ void __launch_bounds__(THR) first_split(const __grid_constant__ SynthArgs a)
+__global__ void __launch_bounds__(THR, 6) first_split(const __grid_constant__ SynthArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     first_split_body(a, blockIdx.x, smem);
 }
 
-__global__ void __launch_bounds__(THR) first_split_batch(const SynthArgs *args, const int *prefix, int np)
+__global__ void __launch_bounds__(THR, 6) first_split_batch(const SynthArgs *args, const int *prefix, int np)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ SynthArgs sa;
