@@ -1149,6 +1149,13 @@ __device__ __forceinline__ void set_entry(BetaEntryF &e, double b, double ib)
     e.pad = 0.f;
 }
 
+// Split plans: the Helmholtz sums' rows (series_tables) behind the b table.
+__device__ __forceinline__ const float *far_rows_f32(const EvalArgs &a)
+{
+    const size_t ne = (size_t)(a.n1hi - a.n1lo + 1) * (a.n2hi - a.n2lo + 1);
+    return reinterpret_cast<const float *>(reinterpret_cast<const BetaEntryF *>(a.btab) + ((ne + 1) & ~(size_t)1));  // 32-byte loads
+}
+
 // Series tables of a 3D plan, built on the device: the b table over the index
 // box, the exponential table e^{-(j - j0)/128}, and (block 0, warp 0) the list
 // of propagating indices in row-major order of the sub-box pbox = [n1lo, n1hi,
@@ -1175,6 +1182,22 @@ __global__ void series_tables(EvalArgs a, E *tab, double2 *exptab, longlong2 *tr
             set_entry(e, b, 1.0 / b);
         }
         tab[i] = e;
+    }
+    if (sizeof(E) == sizeof(BetaEntryF)) {
+        // the Helmholtz sums' rows behind it: by groups of four, -b log2(e) and then -log2 b, padded
+        // with weight 0
+        float *fb = const_cast<float *>(far_rows_f32(a));
+        const int W4 = (W2 + 3) & ~3, rows = a.n1hi - a.n1lo + 1;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows * W4; i += gridDim.x * blockDim.x) {
+            const int r = i / W4, q = i - r * W4;
+            const double c1 = a.a1 + (a.n1lo + r), c2 = a.a2 + (a.n2lo + q);
+            const double aa = sqrt(c1 * c1 + c2 * c2);
+            const bool ev = q < W2 && aa > a.k;
+            const double b = ev ? sqrt((aa - a.k) * (aa + a.k)) : 1.0;
+            float *f = fb + ((size_t)r * W4 + (q & ~3)) * 2 + (q & 3);
+            f[0] = ev ? (float)(-b * 1.4426950408889634) : -CUDART_INF_F;
+            f[4] = ev ? (float)-log2(b) : 0.f;
+        }
     }
     if (exptab)
         for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < a.exptab_n; j += gridDim.x * blockDim.x)
@@ -2287,6 +2310,11 @@ struct FarChunks {
         const int smax = !fp64 ? FAR_SLABS_MAX / 2 : nch <= FAR_LONG ? FAR_SLABS_MAX : FAR_SLABS_LONG;
         return far_slabs_capped(a, kind, (count + 31) >> 5, far_slabs(nch, smax));
     }
+    // the same for items of two chunks
+    __device__ __forceinline__ int slabs2(const EvalArgs &a, int items) const
+    {
+        return far_slabs_capped(a, 0, (count + 31) >> 5, far_slabs(items, FAR_SLABS_MAX / 2, 2));
+    }
 };
 static_assert(GF_FAR_CELLS < 32768, "cells are listed as short");
 
@@ -2408,11 +2436,195 @@ __global__ void __launch_bounds__(128) far3d_tail(EvalArgs a)
 // ex2; the per-target cell reduction and the lattice phase's fractional part in
 // double, everything else in float.
 // ---------------------------------------------------------------------------
-template <int NF>
-__device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, int nslab)
+// Pairs of floats in a 64-bit register: the packed multiply-add issues once for two.
+__device__ __forceinline__ uint64_t pack2(float x, float y)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t ex2x2(uint64_t a)
+{
+    float x, y;
+    unpack2(a, x, y);
+    return pack2(ex2_approx(x), ex2_approx(y));
+}
+
+// Helmholtz sums of H = 1 or 2 chunks of 32 targets (chunk indices w, -1: none), a target of
+// each per lane.
+//
+// A row's evanescent terms: weights e^{-b|x3|}/b = 2^(-b log2(e) |x3| - log2 b) by one multiply-add and ex2 from
+// the rows behind the b table, summed by Horner's rule in v^4, v = e^{i t2}, the even and the odd terms
+// in the halves of packed multiply-adds (eight, four ex2 and one load for four terms).  Issue bounds
+// it, so the loads, the row bounds (formed by one lane per row, 32 rows at a time) and the loops
+// are shared by two targets where the list is long enough.  64 pairs with 2.2 million far targets:
+// term by term with 1/b from the table 2.61 ms, groups 2.21, two targets a lane 1.68 (at 80 registers:
+// with 102 and 16 warps an SM 2.44).  A million targets of one plan (series kernels alone) 605 -> 556 us.
+__device__ __forceinline__ void load_rows(const float *p, uint64_t &b0, uint64_t &b1, uint64_t &l0, uint64_t &l1)
+{
+    const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2 *>(p)), l = __ldg(reinterpret_cast<const ulonglong2 *>(p + 4));
+    b0 = b.x;
+    b1 = b.y;
+    l0 = l.x;
+    l1 = l.y;
+}
+
+template <int H>
+__device__ void far3d_f32_helm(const EvalArgs &a, const int (&w)[H], int count, int slab, int nslab)
+{
+    const int W2 = a.n2hi - a.n2lo + 1, W4 = (W2 + 3) & ~3;
+    const float *frows = far_rows_f32(a);
+    const int lane = threadIdx.x & 31;
+    const float a1f = (float)a.a1, a2f = (float)a.a2, k2f = (float)(a.k * a.k);
+    int idx[H];
+    bool valid[H];
+    double m1[H], m2[H];
+    float z[H], t1[H], t2[H], sv[H], cv[H], Px[H], Py[H], Sx[H], Sy[H];
+    float R2mf = 0.f;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const int slot = w[h] * 32 + lane;
+        valid[h] = w[h] >= 0 && slot < count;
+        idx[h] = valid[h] ? a.far_sorted[slot] : 0;
+        double x1 = 0, x2 = 0, x3 = 1;
+        if (valid[h]) {
+            x1 = a.x[3 * (size_t)idx[h]];
+            x2 = a.x[3 * (size_t)idx[h] + 1];
+            x3 = a.x[3 * (size_t)idx[h] + 2];
+        }
+        // cell reduction by a multiply and a floor: the series is the same for any
+        // decomposition x = 2 pi m + t (e^{i alpha_n . x} = e^{i alpha_n . t}
+        // e^{i 2 pi alpha . m}), so the exact cell decision of the near branch
+        // is not needed here
+        m1[h] = floor(fma(x1, INV_TWO_PI, 0.5));
+        m2[h] = floor(fma(x2, INV_TWO_PI, 0.5));
+        t1[h] = (float)fma(-TWO_PI, m1[h], x1);
+        t2[h] = (float)fma(-TWO_PI, m2[h], x2);
+        z[h] = fabsf((float)x3);
+        const float Tz = (float)a.T / z[h];
+        if (valid[h]) R2mf = fmaxf(R2mf, k2f + Tz * Tz);
+        sincos_cw(t2[h], sv[h], cv[h]);
+        Px[h] = Py[h] = Sx[h] = Sy[h] = 0.f;
+    }
+    for (int o = 16; o > 0; o >>= 1) R2mf = fmaxf(R2mf, __shfl_xor_sync(0xffffffffu, R2mf, o));
+    for (int q = 0, nq = slab == 0 ? *a.nprop : 0; q < nq; ++q) {
+        const PropEntry &pe = a.prop[q];
+        const float br = pe.brf, ibr = pe.ibrf, c1 = pe.c1f, c2 = pe.c2f;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            float sz, cz, sp, cp;
+            sincos_cw(br * z[h], sz, cz);
+            sincos_cw(c1 * t1[h] + c2 * t2[h], sp, cp);
+            Px[h] += ibr * (cz * cp - sz * sp);
+            Py[h] += ibr * (cz * sp + sz * cp);
+        }
+    }
+    uint64_t zz[H], v2x[H], v2y[H], v4x[H], v4y[H], nv4y[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const float q2x = cv[h] * cv[h] - sv[h] * sv[h], q2y = 2.f * cv[h] * sv[h], q4x = q2x * q2x - q2y * q2y,
+                    q4y = 2.f * q2x * q2y;
+        zz[h] = pack2(z[h], z[h]);
+        v2x[h] = pack2(q2x, q2x);
+        v2y[h] = pack2(q2y, q2y);
+        v4x[h] = pack2(q4x, q4x);
+        v4y[h] = pack2(q4y, q4y);
+        nv4y[h] = pack2(-q4y, -q4y);
+    }
+    // row bounds in float with a one-index margin; row slab: the rows split evenly
+    const float Rmf = sqrtf(R2mf);
+    const int n1a = max(a.n1lo, (int)floorf(-a1f - Rmf) - 1), n1b = min(a.n1hi, (int)ceilf(-a1f + Rmf) + 1);
+    const int nr = n1b - n1a + 1;
+    const int r_lo = n1a + (slab * nr) / nslab, r_hi = n1a + ((slab + 1) * nr) / nslab - 1;
+    for (int r0 = r_lo; r0 <= r_hi; r0 += 32) {
+        // groups of four from n2lo on, first and number, of row r0 + lane (the groups at the ends may pass
+        // the truncation: the terms are there and below e^{-T})
+        int gfirst = 0, gnum = 0;
+        {
+            const float c1 = a1f + (float)(r0 + lane), remf = R2mf - c1 * c1, srf = sqrtf(fmaxf(remf, 0.f));
+            const int n2a = max(a.n2lo, (int)floorf(-a2f - srf) - 1), n2b = min(a.n2hi, (int)ceilf(-a2f + srf) + 1);
+            if (remf >= -1.0f && n2a <= n2b && r0 + lane <= r_hi) {
+                gfirst = (n2a - a.n2lo) & ~3;
+                gnum = (((n2b - a.n2lo) & ~3) - gfirst) / 4 + 1;
+            }
+        }
+        for (int r = 0; r < min(32, r_hi - r0 + 1); ++r) {
+            const int g0 = __shfl_sync(0xffffffffu, gfirst, r), ng = __shfl_sync(0xffffffffu, gnum, r);
+            if (ng == 0) continue;
+            const float *rb = frows + (size_t)(r0 + r - a.n1lo) * 2 * W4 + 2 * (g0 + 4 * (ng - 1));
+            uint64_t X[H], Y[H];  // (even, odd) terms' sums
+#pragma unroll
+            for (int h = 0; h < H; ++h) X[h] = Y[h] = 0;
+            auto group = [&](uint64_t B0, uint64_t B1, uint64_t L0, uint64_t L1) {
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    // propagating n (summed separately) have -inf, so weight 0
+                    const uint64_t w01 = ex2x2(fma2(B0, zz[h], L0)), w23 = ex2x2(fma2(B1, zz[h], L1));
+                    const uint64_t x = fma2(w23, v2x[h], w01), y = mul2(w23, v2y[h]);
+                    const uint64_t nX = fma2(X[h], v4x[h], fma2(Y[h], nv4y[h], x));
+                    Y[h] = fma2(X[h], v4y[h], fma2(Y[h], v4x[h], y));
+                    X[h] = nX;
+                }
+            };
+            // two groups a turn, both loads first
+            uint64_t A0, A1, A2, A3, B0, B1, B2, B3;
+            if (ng & 1) {
+                load_rows(rb, A0, A1, A2, A3);
+                group(A0, A1, A2, A3);
+                rb -= 8;
+            }
+#pragma unroll 1
+            for (int g = ng >> 1; g > 0; --g, rb -= 16) {
+                load_rows(rb, A0, A1, A2, A3);
+                load_rows(rb - 8, B0, B1, B2, B3);
+                group(A0, A1, A2, A3);
+                group(B0, B1, B2, B3);
+            }
+            const float c1 = a1f + (float)(r0 + r), c2 = a2f + (float)(a.n2lo + g0);
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                float xe, xo, ye, yo, sp, cp;
+                unpack2(X[h], xe, xo);
+                unpack2(Y[h], ye, yo);
+                const float hx = fmaf(cv[h], xo, fmaf(-sv[h], yo, xe)), hy = fmaf(cv[h], yo, fmaf(sv[h], xo, ye));
+                sincos_cw(c1 * t1[h] + c2 * t2[h], sp, cp);
+                Sx[h] += cp * hx - sp * hy;
+                Sy[h] += cp * hy + sp * hx;
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        if (w[h] < 0) continue;
+        // e^{i 2pi <alpha.m>} (i/8pi^2): the fractional part in double, the phase in float
+        double ph = a.a1 * m1[h] + a.a2 * m2[h];
+        ph -= rint(ph);
+        float sl, cl;
+        sincospif(2.0f * (float)ph, &sl, &cl);
+        const float sc = (float)(1.0 / (8.0 * GF_PI * GF_PI));
+        float2 vals[1];
+        vals[0] = cmulf(make_float2(-sl * sc, cl * sc), make_float2(Px[h] + Sy[h], Py[h] - Sx[h]));
+        far_deposit(a, 0, w[h], slab, nslab, ((count + 31) >> 5) * 32, valid[h], idx[h], 1, vals);
+    }
+}
+
+// Maxwell sums of one chunk of 32 targets.
+__device__ void far3d_f32_maxwell(const EvalArgs &a, int w, int count, int slab, int nslab)
 {
     const BetaEntryF *tab = reinterpret_cast<const BetaEntryF *>(a.btab);
-    float2 *out = reinterpret_cast<float2 *>(a.out);
     const int ne = n_entries(a.which);
     const int W2 = a.n2hi - a.n2lo + 1;
     const int lane = threadIdx.x & 31;
@@ -2442,12 +2654,9 @@ __device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, i
         for (int o = 16; o > 0; o >>= 1) R2mf = fmaxf(R2mf, __shfl_xor_sync(0xffffffffu, R2mf, o));
         float sv, cv;
         sincos_cw(t2, sv, cv);
-        float P[NF][2];
-        float S[NF == 1 ? 1 : 7][2];
+        float P[7][2], S[7][2];
 #pragma unroll
-        for (int e = 0; e < NF; ++e) P[e][0] = P[e][1] = 0.f;
-#pragma unroll
-        for (int e = 0; e < (NF == 1 ? 1 : 7); ++e) S[e][0] = S[e][1] = 0.f;
+        for (int e = 0; e < 7; ++e) P[e][0] = P[e][1] = S[e][0] = S[e][1] = 0.f;
         for (int q = 0, nq = slab == 0 ? *a.nprop : 0; q < nq; ++q) {
             const PropEntry &pe = a.prop[q];
             const float br = pe.brf, ibr = pe.ibrf, c1 = pe.c1f, c2 = pe.c2f;
@@ -2457,15 +2666,13 @@ __device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, i
             float tx = ibr * (cz * cp - sz * sp), ty = ibr * (cz * sp + sz * cp);
             P[0][0] += tx;
             P[0][1] += ty;
-            if (NF > 1) {
-                float b3 = br * sg;
-                float f[6] = {1.f - c1 * c1 * ik2, 1.f - c2 * c2 * ik2, 1.f - b3 * b3 * ik2,
-                              -c1 * c2 * ik2, -c1 * b3 * ik2, -c2 * b3 * ik2};
+            float b3 = br * sg;
+            float f[6] = {1.f - c1 * c1 * ik2, 1.f - c2 * c2 * ik2, 1.f - b3 * b3 * ik2,
+                          -c1 * c2 * ik2, -c1 * b3 * ik2, -c2 * b3 * ik2};
 #pragma unroll
-                for (int e = 0; e < 6; ++e) {
-                    P[1 + e][0] += f[e] * tx;
-                    P[1 + e][1] += f[e] * ty;
-                }
+            for (int e = 0; e < 6; ++e) {
+                P[1 + e][0] += f[e] * tx;
+                P[1 + e][1] += f[e] * ty;
             }
         }
         // row bounds in float with a one-index margin
@@ -2485,27 +2692,23 @@ __device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, i
             if (n2a > n2b) continue;
             const BetaEntryF *row = tab + (size_t)(n1 - a.n1lo) * W2 - a.n2lo;
             float c2 = a2f + (float)n2b;
-            float h[NF == 1 ? 1 : 6][2];
+            float h[6][2];
 #pragma unroll
-            for (int e = 0; e < (NF == 1 ? 1 : 6); ++e) h[e][0] = h[e][1] = 0.f;
+            for (int e = 0; e < 6; ++e) h[e][0] = h[e][1] = 0.f;
             for (int n2 = n2b; n2 >= n2a; --n2, c2 -= 1.0f) {
                 const BetaEntryF be = row[n2];
                 // propagating n (summed separately) have bl2 = +inf, so e = 0; no
                 // per-lane truncation test (terms beyond the lane's set are below e^{-T})
                 const float e = ex2_approx(-be.bl2 * z);
-                float wv[NF == 1 ? 1 : 6];
-                if (NF == 1) {
-                    wv[0] = e * be.ib;
-                } else {
-                    wv[0] = e * be.ib;
-                    wv[1] = c2 * wv[0];
-                    wv[2] = c2 * wv[1];
-                    wv[3] = be.b * e;
-                    wv[4] = e;
-                    wv[5] = c2 * e;
-                }
+                float wv[6];
+                wv[0] = e * be.ib;
+                wv[1] = c2 * wv[0];
+                wv[2] = c2 * wv[1];
+                wv[3] = be.b * e;
+                wv[4] = e;
+                wv[5] = c2 * e;
 #pragma unroll
-                for (int e2 = 0; e2 < (NF == 1 ? 1 : 6); ++e2) {
+                for (int e2 = 0; e2 < 6; ++e2) {
                     const float nx = fmaf(h[e2][0], cv, fmaf(-h[e2][1], sv, wv[e2]));
                     const float ny = fmaf(h[e2][0], sv, h[e2][1] * cv);
                     h[e2][0] = nx;
@@ -2514,32 +2717,27 @@ __device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, i
             }
             float sp, cp;
             sincos_cw(c1 * t1 + (a2f + (float)n2a) * t2, sp, cp);
-            float r[NF == 1 ? 1 : 6][2];
+            float r[6][2];
 #pragma unroll
-            for (int e2 = 0; e2 < (NF == 1 ? 1 : 6); ++e2) {
+            for (int e2 = 0; e2 < 6; ++e2) {
                 r[e2][0] = cp * h[e2][0] - sp * h[e2][1];
                 r[e2][1] = cp * h[e2][1] + sp * h[e2][0];
             }
-            if (NF == 1) {
-                S[0][0] += r[0][0];
-                S[0][1] += r[0][1];
-            } else {
-                const float fxx = 1.f - c1 * c1 * ik2;
-                S[0][0] += r[0][0];
-                S[0][1] += r[0][1];
-                S[1][0] += fxx * r[0][0];
-                S[1][1] += fxx * r[0][1];
-                S[2][0] += r[0][0] - ik2 * r[2][0];
-                S[2][1] += r[0][1] - ik2 * r[2][1];
-                S[3][0] += r[0][0] + ik2 * r[3][0];
-                S[3][1] += r[0][1] + ik2 * r[3][1];
-                S[4][0] += -c1 * ik2 * r[1][0];
-                S[4][1] += -c1 * ik2 * r[1][1];
-                S[5][0] += -c1 * ik2 * r[4][0];
-                S[5][1] += -c1 * ik2 * r[4][1];
-                S[6][0] += -ik2 * r[5][0];
-                S[6][1] += -ik2 * r[5][1];
-            }
+            const float fxx = 1.f - c1 * c1 * ik2;
+            S[0][0] += r[0][0];
+            S[0][1] += r[0][1];
+            S[1][0] += fxx * r[0][0];
+            S[1][1] += fxx * r[0][1];
+            S[2][0] += r[0][0] - ik2 * r[2][0];
+            S[2][1] += r[0][1] - ik2 * r[2][1];
+            S[3][0] += r[0][0] + ik2 * r[3][0];
+            S[3][1] += r[0][1] + ik2 * r[3][1];
+            S[4][0] += -c1 * ik2 * r[1][0];
+            S[4][1] += -c1 * ik2 * r[1][1];
+            S[5][0] += -c1 * ik2 * r[4][0];
+            S[5][1] += -c1 * ik2 * r[4][1];
+            S[6][0] += -ik2 * r[5][0];
+            S[6][1] += -ik2 * r[5][1];
         }
         // e^{i 2pi <alpha.m>} (i/8pi^2): the fractional part in double, the phase in float
         double ph = a.a1 * m1 + a.a2 * m2;
@@ -2548,38 +2746,47 @@ __device__ void far3d_f32_chunk(const EvalArgs &a, int w, int count, int slab, i
         sincospif(2.0f * (float)ph, &sl, &cl);
         const float sc = (float)(1.0 / (8.0 * GF_PI * GF_PI));
         const float2 pre = make_float2(-sl * sc, cl * sc);
-        constexpr int NE = NF == 1 ? 1 : 7;
-        float2 vals[NE];
-        if (NF == 1) {
-            vals[0] = cmulf(pre, make_float2(P[0][0] + S[0][1], P[0][1] - S[0][0]));
-        } else {
+        float2 vals[7];
 #pragma unroll
-            for (int e = 0; e < 6; ++e) {
-                const float *s = S[1 + e];
-                float2 v;
-                if (e < 4)
-                    v = make_float2(P[1 + e][0] + s[1], P[1 + e][1] - s[0]);
-                else
-                    v = make_float2(P[1 + e][0] + sg * s[0], P[1 + e][1] + sg * s[1]);
-                vals[e] = cmulf(pre, v);
-            }
-            vals[NE - 1] = cmulf(pre, make_float2(P[0][0] + S[0][1], P[0][1] - S[0][0]));
+        for (int e = 0; e < 6; ++e) {
+            const float *s = S[1 + e];
+            float2 v;
+            if (e < 4)
+                v = make_float2(P[1 + e][0] + s[1], P[1 + e][1] - s[0]);
+            else
+                v = make_float2(P[1 + e][0] + sg * s[0], P[1 + e][1] + sg * s[1]);
+            vals[e] = cmulf(pre, v);
         }
+        vals[6] = cmulf(pre, make_float2(P[0][0] + S[0][1], P[0][1] - S[0][0]));
         far_deposit(a, 0, w, slab, nslab, ((count + 31) >> 5) * 32, valid, idx, ne, vals);
-        (void)out;
     }
 }
 
+// Chunks per warp of the grid from which a lane takes two targets.
+constexpr int FAR_PAIRS = 1;
+
 template <int NF>
-__global__ void __launch_bounds__(128) far3d_f32(EvalArgs a)
+__global__ void __launch_bounds__(128, NF == 1 ? 6 : 1) far3d_f32(const __grid_constant__ EvalArgs a)
 {
     __shared__ short rejected[GF_FAR_CELLS];
     const FarChunks ch(a, rejected);
-    const int S = ch.slabs(a, 0, false);
     int *ctr = a.far_count + GF_WORK_SLOT;
+    if (NF == 1 && ch.nch >= FAR_PAIRS * (int)(gridDim.x * blockDim.x >> 5)) {
+        const int np = (ch.nch + 1) >> 1, S = ch.slabs2(a, np);
+        for (int t = far_take(ctr, np * S); t >= 0; t = far_take(ctr, np * S)) {
+            const int u = 2 * (t / S);
+            far3d_f32_helm<2>(a, {ch.at(u), u + 1 < ch.nch ? ch.at(u + 1) : -1}, ch.count, t % S, S);
+        }
+        return;
+    }
+    const int S = ch.slabs(a, 0, false);
     for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
         const int w = ch.at(t / S);
-        if (w >= 0) far3d_f32_chunk<NF>(a, w, ch.count, t % S, S);
+        if constexpr (NF > 1) {
+            if (w >= 0) far3d_f32_maxwell(a, w, ch.count, t % S, S);
+        } else if (w >= 0) {
+            far3d_f32_helm<1>(a, {w}, ch.count, t % S, S);
+        }
     }
 }
 
@@ -2590,16 +2797,19 @@ __global__ void __launch_bounds__(128) far3d_f32(EvalArgs a)
 // load stays balanced across pair boundaries.  The taken index only grows, so
 // each warp walks the pair list forward.
 template <typename R, int NF>
-__global__ void far3d_batch(const EvalArgs *args, int np)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && NF == 1 ? 3 : 1) far3d_batch(const EvalArgs *args, int np)
 {
     if (np <= 0) return;
     int tot = 0;
     for (int q = 0; q < np; ++q) tot += (args[q].far_count[0] + 31) >> 5;
-    const int S = far_slabs(tot, sizeof(R) == 8 ? 8 : 4);
+    // split Helmholtz sweeps of some length: items of two chunks
+    const bool pairs = sizeof(R) == 4 && NF == 1 && tot >= FAR_PAIRS * (int)(gridDim.x * blockDim.x >> 5);
+    const int S = pairs ? far_slabs(tot / 2, 4, 2) : far_slabs(tot, sizeof(R) == 8 ? 8 : 4);
     int *ctr = args[0].far_count + GF_WORK_SLOT;
+    auto items = [&](int n) { return (pairs ? (n + 63) >> 6 : (n + 31) >> 5) * S; };
     int p = 0, base = 0;
     int count = args[0].far_count[0];
-    int nit = ((count + 31) >> 5) * S;
+    int nit = items(count);
     for (;;) {
         int t = 0;
         if ((threadIdx.x & 31) == 0) t = atomicAdd(ctr, 1);
@@ -2608,15 +2818,19 @@ __global__ void far3d_batch(const EvalArgs *args, int np)
             base += nit;
             if (++p < np) {
                 count = args[p].far_count[0];
-                nit = ((count + 31) >> 5) * S;
+                nit = items(count);
             }
         }
         if (p >= np) return;
-        const int u = t - base, nch = nit / S;
-        if (sizeof(R) == 8)
+        const int u = t - base, nch = (count + 31) >> 5;
+        if constexpr (sizeof(R) == 8)
             far3d_f64_chunk<NF, true>(args[p], nch - 1 - u / S, count, u % S, S);
+        else if constexpr (NF > 1)
+            far3d_f32_maxwell(args[p], nch - 1 - u / S, count, u % S, S);
+        else if (pairs)
+            far3d_f32_helm<2>(args[p], {nch - 1 - 2 * (u / S), nch - 2 - 2 * (u / S)}, count, u % S, S);
         else
-            far3d_f32_chunk<NF>(args[p], nch - 1 - u / S, count, u % S, S);
+            far3d_f32_helm<1>(args[p], {nch - 1 - u / S}, count, u % S, S);
     }
 }
 

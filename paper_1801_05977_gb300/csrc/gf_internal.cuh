@@ -255,11 +255,11 @@ struct EvalArgs {
 // Targets from which an evaluation takes the product path (uniform targets, |x3| <= 1, times of
 // the whole evaluation, series kernels against products): double Helmholtz 263 / 418 us at 8000
 // (there the cells are too wide in |x3|), 408 / 286 at 16000; double Maxwell 1090 / 1312 at 16000,
-// 1832 / 967 at 32000; split Helmholtz 193 / 216 at 128000, 297 / 277 at 256000; split Maxwell
-// 704 / 714 at 256000, 1264 / 1150 at 512000.
+// 1832 / 967 at 32000; split Helmholtz 356 / 363 at 512000, 556 / 541 at a million (k = 5: 381 / 374, 608 / 555);
+// split Maxwell 704 / 714 at 256000, 1264 / 1150 at 512000.
 inline int64_t gf_far_product_min(int precision, int nf)
 {
-    return precision == GF_FP64 ? (nf == 1 ? 12288 : 20480) : (nf == 1 ? 196608 : 327680);
+    return precision == GF_FP64 ? (nf == 1 ? 12288 : 20480) : (nf == 1 ? 786432 : 327680);
 }
 size_t gf_far_product_bytes(int precision, int64_t n, int nent, int *maxcells);
 cudaError_t gf_launch_far_product(EvalArgs &a, int precision, int nsm, cudaStream_t s);

@@ -658,7 +658,11 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
             if (p->exptab_j0 < S) p->exptab_j0 = S;
             p->exptab_n = p->exptab_j0 + S * ((int)ceil(p->T + log(1.4143 * (Rc + 2.0))) + 2) + 1;
             const bool want_exp = p->precision == GF_FP64;
-            if ((e = gf_dev_alloc(&p->btab, ne * eb, st)) != cudaSuccess ||
+            // split plans: the Helmholtz sums' float rows after it (eval.cu)
+            const size_t fb = p->precision == GF_FP64 ? 0
+                                                      : sizeof(float) * 2 * (size_t)(p->n1hi - p->n1lo + 1) *
+                                                            (size_t)((p->n2hi - p->n2lo + 4) & ~3);
+            if ((e = gf_dev_alloc(&p->btab, ((ne + 1) & ~(size_t)1) * eb + fb, st)) != cudaSuccess ||
                 (e = gf_dev_alloc((void **)&p->prop, sizeof(PropEntry) * nprop_max + 16, st)) != cudaSuccess ||
                 (e = gf_dev_alloc((void **)&p->trig, sizeof(longlong2) * GF_TRIG_STEPS, st)) != cudaSuccess ||
                 (want_exp && (e = gf_dev_alloc((void **)&p->exptab, 2 * sizeof(double2) * p->exptab_n, st)) != cudaSuccess)) {
