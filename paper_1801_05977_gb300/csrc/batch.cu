@@ -132,7 +132,7 @@ static gf_status batch_eval_setup(gf_batch_t b, const double *x, const int64_t *
         ea[p].far_sorted = b->scratch + b->cap + off[p];
         ea[p].near_idx = b->scratch + 2 * b->cap + off[p];
         ea[p].far_count = b->counters + (size_t)GF_SCRATCH_COUNTERS * p;
-        pre[p + 1] = pre[p] + (int)((n + 255) / 256);
+        pre[p + 1] = pre[p] + (int)((n + GF_BATCH_TILE - 1) / GF_BATCH_TILE);
     }
     CUB(cudaMemcpy(b->d_eargs, ea.data(), sizeof(EvalArgs) * b->np, cudaMemcpyHostToDevice));
     CUB(cudaMemcpy(b->d_prefix + 3 * (b->np + 1), pre.data(), sizeof(int) * (b->np + 1), cudaMemcpyHostToDevice));
@@ -141,8 +141,8 @@ static gf_status batch_eval_setup(gf_batch_t b, const double *x, const int64_t *
     b->eb.np = b->np;
     b->eb.nf = b->nf;
     b->eb.grid_near = pre[b->np] < b->nsm * 16 ? (pre[b->np] > 0 ? pre[b->np] : 1) : b->nsm * 16;
-    b->eb.scatter_per_pair = 2;
-    b->eb.grid_scatter = b->np * 2 < b->nsm * 4 ? b->np * 2 : b->nsm * 4;
+    b->eb.scatter_per_pair = 8;
+    b->eb.grid_scatter = std::min(b->np * b->eb.scatter_per_pair, b->nsm * 4);
     b->eb.block_far = b->tune.far_block;
     b->eb.grid_far = b->nsm * b->tune.far_per_sm * 128 / b->tune.far_block;
     b->cur = GraphKey{x, out, which, std::vector<int64_t>(off, off + b->np + 1)};

@@ -144,6 +144,11 @@ struct SynthArgs {
     // 3D split plans: the columns formed in double lie in the box n1 = dbx0 ..
     // dbx0 + dbw - 1, n2 from dby0, ndbl columns in all (0 in other plans)
     int dbx0, dbw, dby0, ndbl;
+    // X' sums of evanescent columns (large double 3D grids, else null): panels of width
+    // xpw in g = |beta|, [xpn][GF_XDEG1][Mlast/2 + 1] (s1, s3) by powers of g - centre, times e^{(centre - g) xptc}
+    const double2 *xp;
+    int xpn;
+    double xpw, ixpw, xptc;
 };
 
 // Complex entries per target of an output selection (gf_eval_points `which`).
@@ -295,9 +300,10 @@ struct SynthBatch {
     int total0;             // virtual blocks of the first pass
     size_t smem[3];
 };
+constexpr int GF_BATCH_TILE = 1024;
 struct EvalBatch {
     const EvalArgs *args;   // per pair: x, out, n and scratch pointers filled in
-    const int *prefix;      // near-kernel tiles (256 targets) per pair, prefix sums (np + 1)
+    const int *prefix;      // classification tiles (GF_BATCH_TILE targets) per pair, prefix sums (np + 1)
     int np;
     int nf;
     int grid_near, grid_scatter, grid_far, block_far;
@@ -306,6 +312,7 @@ struct EvalBatch {
 
 // degree of the panels' interpolants; row length of SynthArgs::Ef
 constexpr int GF_HDEG = 14;
+constexpr int GF_XDEG1 = 12;  // coefficients of a panel of the X' sums
 __host__ __device__ constexpr int GF_EF_ROW(int n) { return ((n >> 1) + 8) & ~7; }
 
 // One panel's polynomial (two real functions packed in a double2) at x in [-1, 1].
@@ -353,6 +360,7 @@ struct NodeTables {
 };
 size_t gf_node_powers(int dim, int Q, bool deriv, double eps);
 cudaError_t gf_launch_node_tables(const NodeTables &a, cudaStream_t s);
+cudaError_t gf_launch_xprime_panels(const NodeTables &a, const double *tW, int npan, double w, double tc, double2 *out, cudaStream_t s);
 cudaError_t gf_launch_panels(const NodeTables &a, int dim, int npan, double2 *out, float2 *outf, double2 *dout, cudaStream_t s);
 // far-region grid: the planes' coefficients into a.work ([nf][L3count][M2][M1], FFT
 // order), then the x2 and x1 passes into a.grid (a.zlinear set)
