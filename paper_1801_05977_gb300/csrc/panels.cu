@@ -47,7 +47,7 @@ constexpr Economy economy()
     }
     return E;
 }
-__constant__ Economy c_econ = economy();
+__device__ const Economy c_econ = economy();
 
 // C(p, j) for p <= 26 (exact), 1/p!.
 struct Binomials {
@@ -67,7 +67,7 @@ constexpr Binomials binomials()
     }
     return B;
 }
-__constant__ Binomials c_bin = binomials();
+__device__ const Binomials c_bin = binomials();
 
 // The sums over the nodes of one 2D panel, (set, order n, power q): set 0 the J0
 // transform (n <= q, n + q even), set 1 the J1 transform (n <= q + 1, n + q odd), set 2 the
@@ -94,7 +94,7 @@ constexpr Combos combos()
 }
 constexpr Combos COMBOS = combos();
 static_assert(COMBOS.n <= 448 && COMBOS.n01 <= 256, "one thread per sum");
-__constant__ Combos c_combos = combos();
+__device__ const Combos c_combos = combos();
 
 // Last-axis phases E[b][m] = e^{i q_b t_m}, q_b = j qs (qs = pi / c~) with j = b for b <
 // Mlast/2, else b - Mlast (the last-axis frequencies of Eq. (fck-coef)), t_m the Gauss nodes
@@ -260,6 +260,39 @@ __device__ void bessel_orders(double u, double *out, int stride)
     }
 }
 
+// X' sums s1, s3 = sum_m W_m e^{-g t_m} (cos, sin)(q_b t_m) of evanescent columns on panels in g: with
+// x = g - cen, e^{-g t} = e^{-x tc} e^{-cen t} e^{-x (t - tc)}, tc the middle of the nodes, and the last factor's
+// Taylor sum to power 11: |x (t - tc)| <= 0.2, remainder below 1e-17.
+constexpr int XB = 16;
+__global__ void __launch_bounds__(XB * GF_XDEG1) xprime_panels(NodeTables a, const double *tW, double w, double tc, double2 *out)
+{
+    extern __shared__ double U[];  // [GF_XDEG1][Q]
+    const double cen = (blockIdx.x + 0.5) * w;
+    const int Q = a.Q, nh = (a.Mlast >> 1) + 1;
+    for (int m = threadIdx.x; m < Q; m += blockDim.x) {
+        const double t = a.tt[m], d = tc - t;
+        double f = tW[m] * exp(-cen * t);
+#pragma unroll
+        for (int k = 0; k < GF_XDEG1; ++k) {
+            U[k * Q + m] = f * c_bin.ifact[k];
+            f *= d;
+        }
+    }
+    __syncthreads();
+    const int k = threadIdx.x / XB, b = blockIdx.y * XB + threadIdx.x % XB;
+    if (b >= nh) return;
+    const double2 *E = a.E + (size_t)b * Q;
+    const double *u = U + k * Q;
+    double s1[2] = {0.0, 0.0}, s3[2] = {0.0, 0.0};
+#pragma unroll 8
+    for (int m = 0; m < Q; ++m) {
+        const double2 e = __ldg(E + m);
+        s1[m & 1] = fma(u[m], e.x, s1[m & 1]);
+        s3[m & 1] = fma(u[m], e.y, s3[m & 1]);
+    }
+    out[((size_t)blockIdx.x * GF_XDEG1 + k) * nh + b] = make_double2(s1[0] + s1[1], s3[0] + s3[1]);
+}
+
 constexpr int NC = 128;       // nodes per chunk
 constexpr int LD = NC + 1;    // row length in shared memory (conflict-free columns)
 
@@ -377,6 +410,17 @@ cudaError_t gf_launch_node_tables(const NodeTables &a, cudaStream_t s)
     int blocks = (a.Mlast * a.Q + 127) / 128;
     if (blocks > 1024) blocks = 1024;
     node_tables<<<blocks, 128, 0, s>>>(a);
+    gf_count_launch(1);
+    return cudaGetLastError();
+}
+
+cudaError_t gf_launch_xprime_panels(const NodeTables &a, const double *tW, int npan, double w, double tc, double2 *out, cudaStream_t s)
+{
+    const size_t sm = sizeof(double) * GF_XDEG1 * a.Q;
+    cudaError_t e = cudaFuncSetAttribute(xprime_panels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const int nh = (a.Mlast >> 1) + 1;
+    xprime_panels<<<dim3(npan, (nh + XB - 1) / XB), XB * GF_XDEG1, sm, s>>>(a, tW, w, tc, out);
     gf_count_launch(1);
     return cudaGetLastError();
 }

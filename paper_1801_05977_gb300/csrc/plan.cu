@@ -446,7 +446,17 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
     const bool ftabs = dim == 3 && tr.precision == GF_FP32_SPLIT;  // float copies for the split plans' coefficients
     const size_t dcheb_n = deriv ? 3 * hcheb_n : 0;
     const size_t npow = gf_node_powers(dim, Q, deriv, eps), npow2 = (npow + 1) / 2;
-    const size_t tab_bytes = host_tab_bytes + sizeof(double2) * (E_n + hcheb_n + dcheb_n + npow2) +
+    // smallest g with e^{-g c}/(2 g^2) < 1e-20 (the function decreases in g): beyond it a column's X' integrals
+    // are not formed
+    double gskip = 1.0;
+    while (exp(-gskip * c) / (2.0 * gskip * gskip) >= 1e-20) gskip += 0.25;
+    // X' panels: worth their tables (about 200 columns' sums) on the double 3D plans' grids from 1024
+    // columns on (128 x 128 x 64: the first pass 300 -> 205 us, their tables 18)
+    const double xpw = 0.4 / (0.25 * (ct - c));
+    const int xpn = (int)fmin(ceil(gskip / xpw), 1e6);
+    const bool xpan = dim == 3 && tr.precision == GF_FP64 && M[0] * M[1] >= 1024 && xpn <= 64;
+    const size_t xp_n = xpan ? (size_t)xpn * GF_XDEG1 * (Mlast / 2 + 1) : 0;
+    const size_t tab_bytes = host_tab_bytes + sizeof(double2) * (E_n + hcheb_n + dcheb_n + npow2 + xp_n) +
                              (ftabs ? sizeof(float2) * (E_n + hcheb_n) : 0);
     const size_t work_bytes = gf_plan_work_bytes(p);
     void *work = nullptr;
@@ -470,7 +480,8 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
         double *d_rrd = (double *)(d_B + Q), *d_wyd = d_rrd + (deriv ? 2 * Q : 0);
         double2 *d_E = (double2 *)(d_wyd + (deriv ? 2 * Q : 0)), *d_H = d_E + E_n, *d_D = d_H + hcheb_n;
         double2 *d_pow = d_D + dcheb_n;
-        float2 *d_Ef = ftabs ? (float2 *)(d_pow + npow2) : nullptr, *d_Hf = ftabs ? d_Ef + E_n : nullptr;
+        double2 *d_xp = d_pow + npow2;
+        float2 *d_Ef = ftabs ? (float2 *)(d_xp + xp_n) : nullptr, *d_Hf = ftabs ? d_Ef + E_n : nullptr;
         {
             std::vector<char> pack(host_tab_bytes, 0);
             char *hb = pack.data();
@@ -500,7 +511,8 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
             nt.Bp = npow && dim == 3 ? d_pow : nullptr;
             nt.W = npow && dim == 2 ? (double *)d_pow : nullptr;
             if ((e = gf_stage_upload(tb, hb, host_tab_bytes, st)) == cudaSuccess && (e = gf_launch_node_tables(nt, st)) == cudaSuccess) {
-                if (npow)
+                if (xpan && (e = gf_launch_xprime_panels(nt, d_tW, xpn, xpw, 0.5 * (c + cm), d_xp, st)) != cudaSuccess) {
+                } else if (npow)
                     e = gf_launch_panels(nt, dim, hnpan, d_H, d_Hf, d_D, st);
                 else if ((e = gf_launch_cheb_table(dim, d_rr, d_B, d_P0, d_P1, Q, hnpan, hdeg, hpan, d_H, d_Hf, st)) == cudaSuccess && deriv)
                     e = gf_launch_cheb_deriv(d_rrd, d_wyd, 2 * Q, hnpan, hdeg, hpan, d_D, st);
@@ -527,12 +539,12 @@ gf_status gf_plan(int dim, double k, const double *alpha, const int *M, const gf
         sa.qs = GF_PI / ct;
         sa.qsh = (float)sa.qs;
         sa.qsl = (float)(sa.qs - (double)sa.qsh);
-        // smallest g with e^{-g c}/(2 g^2) < 1e-20 (the function decreases in g)
-        {
-            double g = 1.0;
-            while (exp(-g * c) / (2.0 * g * g) >= 1e-20) g += 0.25;
-            sa.gskip = g;
-        }
+        sa.gskip = gskip;
+        sa.xp = xpan ? d_xp : nullptr;
+        sa.xpn = xpn;
+        sa.xpw = xpw;
+        sa.ixpw = 1.0 / xpw;
+        sa.xptc = 0.5 * (c + cm);
         sa.invV = dim == 3 ? 1.0 / (8.0 * GF_PI * GF_PI * ct) : 1.0 / (4.0 * GF_PI * ct);
         sa.tW = d_tW;
         sa.tt = d_tt;

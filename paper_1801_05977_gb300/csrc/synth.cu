@@ -35,11 +35,28 @@ __device__ __forceinline__ double2 beta_of(double k, double a2)
 // s1 - i s3, I2 = s1 + i s3 and T1 - T2 = (g s1 - q s3)/(g (g^2 + q^2)); for g >
 // gskip both terms are below double rounding of the coefficient (|I| <= e^{-g c},
 // |2 beta (q -+ beta)| >= 2 g^2) and are not formed.
-__device__ __forceinline__ double2 xprime_terms(double2 beta, double q, const double2 *Am, const double2 *Em, int Q,
+//
+// With panels (a.xp: large 3D grids), the evanescent sums come from them: s1 and s3 are e^{-x tc} times a
+// polynomial in x = g - (panel centre) for each b, Am holding x, e^{-x tc} and the panel
+// (24 multiply-adds for 128 with 64 nodes, and no e^{-g t_m} to form).
+__device__ __forceinline__ double2 xprime_terms(const SynthArgs &a, double2 beta, double q, const double2 *Am, int b, int Q,
                                                 double gskip)
 {
+    const double2 *Em = a.E + (size_t)b * Q;
     double2 T12 = make_double2(0.0, 0.0);
-    if (beta.y > 0.0 && beta.y <= gskip) {
+    if (beta.y > 0.0 && beta.y <= gskip && a.xp) {
+        const double x = Am[0].x, e = Am[0].y, g = beta.y;
+        const int nh = (a.Mlast >> 1) + 1;
+        const double2 *c = a.xp + (size_t)__double2loint(Am[1].x) * GF_XDEG1 * nh + b;
+        double2 v = c[(GF_XDEG1 - 1) * nh];
+#pragma unroll
+        for (int k = GF_XDEG1 - 2; k >= 0; --k) {
+            const double2 ck = c[k * nh];
+            v.x = fma(v.x, x, ck.x);
+            v.y = fma(v.y, x, ck.y);
+        }
+        T12.x = e * (g * v.x - q * v.y) / (g * (g * g + q * q));
+    } else if (beta.y > 0.0 && beta.y <= gskip) {
         double s1 = 0.0, s3 = 0.0;
         for (int m = 0; m < Q; ++m) {
             const double A = Am[m].x;
@@ -196,7 +213,7 @@ __device__ void load_twiddles(typename cplx_t<R>::T *tw, int n)
 template <typename C>
 __device__ void deriv_fields_2d(const SynthArgs &a, C *buf0, int TJ, int t, int n, int b, int jx, double q,
                                 double eta, double F1, double S1, double2 K, double A2, const double2 *Am2,
-                                const double2 *Em, double2 beta2, int pnl, double x)
+                                double2 beta2, int pnl, double x)
 {
     typedef decltype(C().x) R;
     const double ip = 2.0 * GF_PI, al = a.a1, kk = a.k * a.k, c1 = al + jx;
@@ -228,7 +245,7 @@ __device__ void deriv_fields_2d(const SynthArgs &a, C *buf0, int TJ, int t, int 
     buf0[(2 * TJ + t) * n + b] = cmk((R)(-q * K.y * sc), (R)((q * K.x - H2i) * sc));
     if (a.nf < 6) return;
     const double dk2 = kk - a.k2 * a.k2;
-    const double2 T12 = xprime_terms(beta2, q, Am2, Em, a.Q, a.gskip);
+    const double2 T12 = xprime_terms(a, beta2, q, Am2, b, a.Q, a.gskip);
     const double iD2 = 1.0 / (A2 + q * q - a.k2 * a.k2);
     const double2 dK = make_double2(K.x - (iD2 + T12.x), K.y - T12.y);
     const double base = -0.5 * ip * F1 - 0.5 * al * ip * f2i;  // P0/2 - (i alpha/2) P1c
@@ -288,6 +305,15 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
         int t = i / Q, m = i - t * Q;
         double2 b = betas[t];
         if (b.y > a.gskip) continue;  // this column's X'-integrals are not used
+        if (a.xp && b.y > 0.0) {
+            if (m == 0) {
+                const int pnl = min((int)(b.y * a.ixpw), a.xpn - 1);
+                const double x = b.y - (pnl + 0.5) * a.xpw;
+                Av[i] = make_double2(x, exp(-x * a.xptc));
+                Av[i + 1].x = __hiloint2double(0, pnl);
+            }
+            continue;
+        }
         double tm = a.tt[m];
         double2 e;
         if (b.y == 0.0) {
@@ -335,8 +361,7 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
         double q = (double)jl * a.qs;
         double A2 = A2s[t];
         const double2 *Am = Av + t * Q;
-        const double2 *Em = a.E + (size_t)b * Q;
-        const double2 T12 = xprime_terms(beta, q, Am, Em, Q, a.gskip);
+        const double2 T12 = xprime_terms(a, beta, q, Am, b, Q, a.gskip);
         double D = A2 + q * q - k2;
         double2 Cj;
         if (a.dim == 3) {
@@ -369,11 +394,11 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
                 F1 = make_double2((1.0 + S0) / eta2, 0.0);
                 // F2 = (-2 i j1 F1 + Phi2-hat/(2 pi))/eta^2,  Phi2-hat/(2 pi) = -i (j1/eta) S1
                 F2 = make_double2(0.0, (-2.0 * jx * F1.x - ((double)jx / eta) * S1) / eta2);
-                if (DERIV) deriv_fields_2d(a, buf0, TJ, t, n, b, jx, q, eta, F1.x, S1, K, A2, Av2 + t * Q, Em,
+                if (DERIV) deriv_fields_2d(a, buf0, TJ, t, n, b, jx, q, eta, F1.x, S1, K, A2, Av2 + t * Q,
                                              need_k2 ? betas2[t] : make_double2(0.0, 0.0), pnl, x);
             }
             if (DERIV && eta2 == 0.0) deriv_fields_2d(a, buf0, TJ, t, n, b, jx, q, 0.0, F1.x, 0.0, K, A2, Av2 + t * Q,
-                                                        Em, need_k2 ? betas2[t] : make_double2(0.0, 0.0), 0, -1.0);
+                                                        need_k2 ? betas2[t] : make_double2(0.0, 0.0), 0, -1.0);
             // C = K - F1 + i alpha F2
             Cj = make_double2(K.x - F1.x - a.a1 * F2.y, K.y - F1.y + a.a1 * F2.x);
             if (DERIV) {
