@@ -2315,8 +2315,10 @@ __device__ __forceinline__ int far_take(int *counter, int nitems)
 // Row slabs per chunk at most.  A short list leaves the GPU empty unless its chunks are cut
 // into single rows (1017 targets: far3d_f64 378 us with 8 slabs, 90 us with 32); from about
 // 300 chunks on the slabs' repeated set-up costs more (13000 far targets: 559 us for
-// the evaluation with 8 slabs, 681 us with 32).  The float sums' set-up is cheap.
-constexpr int FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_LONG = 300;
+// the evaluation with 8 slabs, 681 us with 32).  Up to some 24 chunks even single rows pay (whole
+// evaluations with 32 / 64 / 128 slabs: 1017 targets 146 / 132 / 131 us, 3000 targets 153 / 159 / 177).
+// The float sums' set-up is cheap, their rows short: half as many.
+constexpr int FAR_SLABS_SHORT = 64, FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_SHORT = 24, FAR_LONG = 300;
 
 // Chunks of a far launch: all of the list, or those of the cells that the product
 // path left over (a.rej: their number, tiles per cell, a flag per cell).  The t-th
@@ -2362,7 +2364,8 @@ struct FarChunks {
     // row slabs per chunk: by the chunks of this launch, capped by the scratch of the whole list
     __device__ __forceinline__ int slabs(const EvalArgs &a, int kind, bool fp64) const
     {
-        const int smax = !fp64 ? FAR_SLABS_MAX / 2 : nch <= FAR_LONG ? FAR_SLABS_MAX : FAR_SLABS_LONG;
+        const int s = nch <= FAR_SHORT ? FAR_SLABS_SHORT : nch <= FAR_LONG || !fp64 ? FAR_SLABS_MAX : FAR_SLABS_LONG;
+        const int smax = fp64 ? s : s / 2;
         return far_slabs_capped(a, kind, (count + 31) >> 5, far_slabs(nch, smax));
     }
     // the same for items of two chunks
@@ -2590,8 +2593,11 @@ __device__ void far3d_f32_helm(const EvalArgs &a, const int (&w)[H], int count, 
     uint64_t zz[H], v2x[H], v2y[H], v4x[H], v4y[H], nv4y[H];
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-        const float q2x = cv[h] * cv[h] - sv[h] * sv[h], q2y = 2.f * cv[h] * sv[h], q4x = q2x * q2x - q2y * q2y,
-                    q4y = 2.f * q2x * q2y;
+        // v^2 and v^4 from their own angles: v^4 carries one rounding to the power n/4 where products of v would carry
+        // four
+        float q2x, q2y, q4x, q4y;
+        sincos_cw(2.f * t2[h], q2y, q2x);
+        sincos_cw(4.f * t2[h], q4y, q4x);
         zz[h] = pack2(z[h], z[h]);
         v2x[h] = pack2(q2x, q2x);
         v2y[h] = pack2(q2y, q2y);
@@ -2655,9 +2661,15 @@ __device__ void far3d_f32_helm(const EvalArgs &a, const int (&w)[H], int count, 
                 unpack2(X[h], xe, xo);
                 unpack2(Y[h], ye, yo);
                 const float hx = fmaf(cv[h], xo, fmaf(-sv[h], yo, xe)), hy = fmaf(cv[h], yo, fmaf(sv[h], xo, ye));
-                sincos_cw(c1 * t1[h] + c2 * t2[h], sp, cp);
-                Sx[h] += cp * hx - sp * hy;
-                Sy[h] += cp * hy + sp * hx;
+                // the row's phase with the roundings of its argument (up to 200) put back: they were most of the
+                // sum's error (split evaluations against 64 bits: 1.2e-6 where term by term had 1.0e-6; with this and
+                // the powers above 0.52e-6 against 0.86e-6)
+                const float p1 = c1 * t1[h], p2 = c2 * t2[h], ps = p1 + p2, pb = ps - p1;
+                const float lo = ((p1 - (ps - pb)) + (p2 - pb)) + fmaf(c1, t1[h], -p1) + fmaf(c2, t2[h], -p2);
+                sincos_cw(ps, sp, cp);
+                const float sq = fmaf(cp, lo, sp), cq = fmaf(-sp, lo, cp);
+                Sx[h] += cq * hx - sq * hy;
+                Sy[h] += cq * hy + sq * hx;
             }
         }
     }
