@@ -55,9 +55,8 @@ FF_TERM_FLOPS = 98
 TAIL_TERM_FLOPS = 14
 FAR_CORE_Y0 = 18.0
 FAR_FF_GAP = 8.0
-# DRAM bytes of one far3d_f64 launch on this workload: ncu (dram__bytes_read.sum
-# + dram__bytes_write.sum) of a 2e5-target launch, scaled by the far targets
-FAR_TRAFFIC_BYTES = 9.309696e6 * 5
+# DRAM bytes of the far phase on this workload from ncu, or None: not taken for the products
+FAR_TRAFFIC_BYTES = None
 # unit-count peaks, reported beside the measured ones (152 SMs, 2.07 GHz):
 # FP64 2 FMA/clk/SM, FP32 128 FMA/clk/SM
 # in-plane points of the far-region grid of the split leg that uses it
@@ -447,8 +446,8 @@ def run_gpu(args):
     clocks = clk.summary()
     e2e_s = max_over_ranks([np.mean(e2e_t) if e2e_t else float("nan")], dev)[0]
 
-    # roofline of the dominant kernels (the far series of the double-precision plan:
-    # far3d_f64 and its concurrent float-tail kernel far3d_tail), two pipes
+    # the far series' terms at the two ALU pipes' rates (what far3d_f64 and far3d_tail run; long
+    # lists go to the tensor cores instead)
     far_ms = float(np.mean([p[3] for p in ph64]))
     near_ms = float(np.mean([p[2] for p in ph64]))
     synth_ms = float(np.mean([p[0] for p in ph64]))
@@ -528,7 +527,7 @@ def run_gpu(args):
                            "phases_ms": {"synthesis": float(np.mean([p[0] for p in phfg])),
                                          "near_and_far_grid": float(np.mean([p[2] for p in phfg])),
                                          "far_series": float(np.mean([p[3] for p in phfg]))}},
-        "roofline": {"bound": "alu", "kernel": "far3d_f64 + far3d_tail (concurrent)", "achieved": achieved,
+        "roofline": {"bound": "alu", "kernel": "far series terms (far_product from 12288 targets, else far3d_f64 + far3d_tail)", "achieved": achieved,
                      "peak": peaks["fp64"], "unit": "TFLOP/s (FP64-equivalent)", "frac": achieved / peaks["fp64"],
                      "traffic": FAR_TRAFFIC_BYTES if n_targets == 1_000_000 and FAR_TRAFFIC_BYTES else None,
                      "peaks_measured": {"fp64_tflops": peaks["fp64"], "fp32_tflops": peaks["fp32"],
@@ -544,7 +543,9 @@ def run_gpu(args):
                              "flops + FP32 term flops x P64/P32) / far-phase time, peak = measured FP64 rate, so "
                              "frac = W64/(P64 t) + W32/(P32 t); per term 14 FP64 flops (double band), 98 FP32 "
                              "flops (float-float band), 14 FP32 flops (float tail); frac_max_model takes the "
-                             "busier pipe alone"},
+                             "busier pipe alone.  Long lists sum these terms as matrix products on the tensor "
+                             "cores, off both pipes: the fraction is then a speed in units of the series "
+                             "kernels' bound and may exceed 1"},
         "err_vs_oracle": err_oracle,
         "e2e": {"value": whole_job_rate(n_targets, world, e2e_s), "unit": "evals/s",
                 "h2d_bytes_per_step": int(x_np.nbytes), "d2h_bytes_per_step": int(n_targets * 16)},

@@ -366,7 +366,7 @@ __device__ void synth_first_pass_body(const SynthArgs &a, int blk, unsigned char
         double2 Cj;
         if (a.dim == 3) {
             // h(s) = sum_m B_m sin(s r_m)/s, read from its piecewise Chebyshev
-            // interpolant (Clenshaw); h has bandwidth 2 eps in s, so degree 14 on
+            // interpolant (Horner); h has bandwidth 2 eps in s, so degree 14 on
             // panels of width 2 reproduces the quadrature to rounding.
             double s = sqrt(A2 + q * q);
             int pnl = min((int)(s * a.ihpan), a.hnpan - 1);
@@ -927,6 +927,7 @@ __device__ __forceinline__ double to_power(const double *c, int stride, int t)
     return s;
 }
 
+// Plans with 2 eps > 1 (the others: panels.cu).
 // Piecewise Chebyshev interpolants of the radial transforms, one CTA per panel
 // [p w, (p+1) w]: values at the nn <= 16 Chebyshev points (sixteen threads per
 // point share the quadrature sum, reduced by shuffles), then the discrete
