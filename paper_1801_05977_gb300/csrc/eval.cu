@@ -2981,8 +2981,9 @@ __device__ __forceinline__ double2 ei_beta(double kk, double c1)
     return make_double2(aa > kk ? b : -b, 1.0 / b);
 }
 
-// e^{-y}, y >= 0 (else of no use, but finite): y = j/64 + r, |r| <= 1/128, T[j] = e^{-j/64};
-// truncation r^7/5040 < 4e-19.
+// e^{-y}, y >= 0: y = j/64 + r, |r| <= 1/128, T[j] = e^{-j/64}; truncation r^7/5040 < 4e-19.
+// Propagating indices come with y = -|beta||x2| and discard the result; from 2^25 on the
+// low word of their j has wrapped to any value, so the index is bounded on both sides.
 __device__ __forceinline__ double exp_neg_tab(double y, const double *T)
 {
     const double w = fma(y, (double)F2_S, 6755399441055744.0);
@@ -2994,7 +2995,7 @@ __device__ __forceinline__ double exp_neg_tab(double y, const double *T)
     p = fma(p, r, -1.0 / 6.0);
     p = fma(p, r, 0.5);
     p = fma(p, r, -1.0);
-    const double t = T[max(j, 0)];
+    const double t = T[min(max(j, 0), F2_Y * F2_S)];
     return fma(t, p * r, t);
 }
 
