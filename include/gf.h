@@ -351,6 +351,15 @@ gf_status gf_mlp_gradients(gf_mlp_t mlp, const float *dev_in, const float *dev_t
                            float *host_loss, void *cuda_stream);
 /* Tensor-core error word (1 after a bounded wait ran out): GF_ERR_TIMEOUT if set. */
 gf_status gf_mlp_error_word(gf_mlp_t mlp, int *out);
+/* Self-test of the training pass's bounded waits (diagnostic): runs the forward and
+ * data-gradient pass of gf_mlp_gradients once, the wait of warp `warp` (0 .. 15; -1:
+ * none) of its first CTA for that CTA's product `step` (seven per 128 rows) taken as
+ * run out.  No parameter or gradient changes.  Synchronises; GF_ERR_TIMEOUT when a
+ * wait ran out (the error word is cleared again, the context stays usable; takes a
+ * few seconds, the waits' limit), GF_OK when none did.  Errors: GF_ERR_ARG
+ * (also with the error word set already), GF_ERR_NOMEM, GF_ERR_CUDA. */
+gf_status gf_mlp_wait_selftest(gf_mlp_t mlp, const float *dev_in, const float *dev_target, int n, int warp, int step,
+                               void *cuda_stream);
 /* G_d at near targets (|x3| <= c) of many (alpha, k) pairs, with the network
  * standing in for the interpolated remainder: G = e^{i2pi<alpha.m>}(e^{i alpha.t}
  * scale*MLP + e^{ikr} Y_eps/(4 pi r)).  Pairs whose Wood distance

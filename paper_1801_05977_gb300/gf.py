@@ -54,7 +54,7 @@ EXPORTS = ["gf_trunc_default", "gf_plan", "gf_eval_grid", "gf_grid_bytes", "gf_e
            "gf_gemm_bf16", "gf_mlp_create", "gf_mlp_param_count", "gf_mlp_params", "gf_mlp_set_scale",
            "gf_mlp_forward", "gf_mlp_train_step", "gf_mlp_gradients", "gf_mlp_error_word", "gf_surrogate_eval",
            "gf_mlp_destroy", "gf_release_memory", "gf_peak_probe", "gf_surrogate_eval_residual",
-           "gf_wait_selftest", "gf_plan_status"]
+           "gf_wait_selftest", "gf_plan_status", "gf_mlp_wait_selftest"]
 
 NOALLOC_MAX_TARGETS = 1 << 18
 
@@ -102,6 +102,7 @@ def lib(build_if_missing: bool = True):
     L.gf_mlp_train_step.argtypes = [vp, vp, vp, i32, ctypes.c_float, vp, vp]
     L.gf_mlp_gradients.argtypes = [vp, vp, vp, i32, vp, vp, vp]
     L.gf_mlp_error_word.argtypes = [vp, P(ctypes.c_int)]
+    L.gf_mlp_wait_selftest.argtypes = [vp, vp, vp, i32, i32, i32, vp]
     L.gf_surrogate_eval.argtypes = [vp, i32, P(d), P(d), P(ctypes.c_int64), vp, vp, d, P(Trunc), P(ctypes.c_int), vp]
     L.gf_surrogate_eval_residual.argtypes = [vp, i32, P(d), P(d), P(ctypes.c_int64), vp, vp, vp, d, P(Trunc),
                                              P(ctypes.c_int), vp]
@@ -125,7 +126,7 @@ def lib(build_if_missing: bool = True):
                  "gf_mlp_forward", "gf_mlp_train_step", "gf_mlp_gradients", "gf_mlp_error_word",
                  "gf_surrogate_eval", "gf_mlp_destroy",
                  "gf_plan_get_info", "gf_destroy", "gf_set_phase_timing", "gf_plan_phase_ms", "gf_release_memory",
-                 "gf_peak_probe", "gf_surrogate_eval_residual", "gf_wait_selftest", "gf_plan_status"):
+                 "gf_peak_probe", "gf_surrogate_eval_residual", "gf_wait_selftest", "gf_plan_status", "gf_mlp_wait_selftest"):
         getattr(L, name).restype = ctypes.c_int
     _lib = L
     return L
@@ -432,6 +433,11 @@ class MLP:
         _check(lib().gf_mlp_gradients(self._h, ctypes.c_void_p(inp.data_ptr()), ctypes.c_void_p(target.data_ptr()),
                                       inp.shape[0], g.ctypes.data, ctypes.byref(loss), _stream_ptr(stream)))
         return g, loss.value
+
+    def wait_selftest(self, inp, target, warp: int, step: int, stream=None) -> int:
+        """gf_mlp_wait_selftest: the status of one training pass in which a wait counts as run out."""
+        return int(lib().gf_mlp_wait_selftest(self._h, ctypes.c_void_p(inp.data_ptr()), ctypes.c_void_p(target.data_ptr()),
+                                              inp.shape[0], int(warp), int(step), _stream_ptr(stream)))
 
     def error_word(self) -> int:
         v = ctypes.c_int()
