@@ -397,6 +397,17 @@ gf_status gf_mlp_destroy(gf_mlp_t mlp);
  * GF_OK otherwise.  Errors: GF_ERR_ARG, GF_ERR_CUDA. */
 gf_status gf_plan_status(gf_plan_t plan, void *cuda_stream);
 
+/* Self-test of the bounded waits of the far series' matrix products (diagnostic):
+ * as gf_eval_points, but the wait of one warp of the products' first CTA counts as
+ * run out: warp 0 (copies) or 1 .. 3 (MMAs) at its `unit`-th hand-over, warp 4 (one of
+ * those that finish the sums) at its `unit`-th pass; unit -1: none.  Synchronises;
+ * GF_ERR_TIMEOUT when a wait ran out (the plan's error word is cleared again, the
+ * context stays usable, dev_out is not to be used; takes a few seconds, the
+ * waits' limit), GF_OK when none did (also where the call does not take the products).
+ * Errors: as gf_eval_points; GF_ERR_ARG also with the error word set already. */
+gf_status gf_eval_wait_selftest(gf_plan_t plan, const double *dev_xyz, int64_t n, int which, void *dev_out, int warp,
+                                int unit, void *cuda_stream);
+
 /* Plan facts (host memory).  Returns GF_ERR_ARG on NULL arguments. */
 typedef struct {
     int dim, M[3], nfields, precision, kind;

@@ -950,8 +950,9 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
     Cell *cell = reinterpret_cast<Cell *>(cmd0 + NMW * (2 * MAXST + 4));
     uint64_t *bars = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(cell) + SM::CELL);
     // A unit written; B unit landed; A, B unit multiplied (an arrival per issuing warp); pass done; accumulators read
-    uint64_t *afull = bars, *bfull = bars + 2, *afree = bars + 4, *bfree = bars + 6, *accf = bars + 8, *tfree = bars + 9;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 10);
+    // and, after a wait that ran out, an issuing warp's MMAs
+    uint64_t *afull = bars, *bfull = bars + 2, *afree = bars + 4, *bfree = bars + 6, *accf = bars + 8, *tfree = bars + 9, *mdone = bars + 10;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 10 + NMW);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int count = a.far_count[0], ntiles = (count + TILE - 1) / TILE, T = rej[1];
@@ -961,8 +962,8 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (threadIdx.x == 0) {
-        for (int q = 0; q < 10; ++q) {
-            const int n = (q < 2 || q == 9) ? NGW : (q < 4 ? 1 : NMW);
+        for (int q = 0; q < 10 + NMW; ++q) {
+            const int n = (q < 2 || q == 9) ? NGW : (q < 4 || q > 9 ? 1 : NMW);
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(umma::smem_u32(&bars[q])), "r"(n));
         }
         *abort_flag = 0;
@@ -976,6 +977,8 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
     int ga = 0, gu = 0, gp = 0;            // A units, B units and passes so far (barrier phases)
     int cur = -1;                          // cell held in shared memory
     bool ok = true;
+    // self-test: the unit (copies, MMAs) or the pass (a warp that finishes sums) whose wait counts as run out
+    const int drop = blockIdx.x == 0 && warp == (a.drop_warp < 4 ? NGW + a.drop_warp : 0) ? a.drop_unit - 1 : -1;
     // After a wait that ran out every warp still takes part in the barriers of its tile;
     // the whole CTA leaves at the next tile.
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -1035,7 +1038,10 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
                         const int t1 = pass == 2 ? cell->pust[u - q * npu + 1] : cell->ust[u + 1];
                         if (w < 0) {
                             if (gu >= SM::NBUF) ok = umma::mbar_wait_sleep(umma::smem_u32(&bfree[buf]), ph ^ 1) && !*abort_flag;
-                            if (!ok) break;
+                            if (!ok || gu == drop) {
+                                ok = false;
+                                break;
+                            }
                             const Stage &S0 = cell->st[t0], &S1 = cell->st[t1 - 1];
                             const int ub = S1.off + S1.img - S0.off, up = S1.poff + S1.pimg - S0.poff;
                             const int bytes = L == 3 ? 2 * ub : pass == 2 ? up : ub;
@@ -1058,7 +1064,7 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
                             }
                         } else {
                             ok = (again || umma::mbar_wait_sleep(umma::smem_u32(&afull[abuf]), (au / SM::NBUF) & 1)) &&
-                                 umma::mbar_wait_sleep(umma::smem_u32(&bfull[buf]), ph) && !*abort_flag;
+                                 umma::mbar_wait_sleep(umma::smem_u32(&bfull[buf]), ph) && !*abort_flag && gu != drop;
                             if (!ok) break;
                             asm volatile("tcgen05.fence::after_thread_sync;");
                             const uint32_t a16 = umma::smem_u32(sA + abuf * SM::A_BYTES) >> 4, b16 = umma::smem_u32(sB + buf * UBYTES) >> 4;
@@ -1143,7 +1149,7 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
                 ++ga;
             };
             auto pass_begin = [&]() {
-                if (ok) ok = __all_sync(0xffffffffu, umma::mbar_wait_sleep(umma::smem_u32(accf), gp & 1) && !*abort_flag);
+                if (ok) ok = __all_sync(0xffffffffu, umma::mbar_wait_sleep(umma::smem_u32(accf), gp & 1) && !*abort_flag) && gp != drop;
                 asm volatile("tcgen05.fence::after_thread_sync;");
             };
             auto pass_end = [&]() {
@@ -1426,10 +1432,17 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
             }
         }
     }
-    // before the CTA exits, copies in flight land (after a wait that ran out; otherwise the last
-    // pass's accumulators, which every copy and MMA precedes, have been read)
-    if (warp == NGW && lane == 0 && !ok)
-        for (int g = max(0, gu - 1); g < gu + 1; ++g) umma::mbar_wait_n(umma::smem_u32(&bfull[g % SM::NBUF]), (g / SM::NBUF) & 1, 1 << 16);
+    // After a wait that ran out anywhere: before the CTA exits, copies in flight (of the last NBUF units
+    // issued, gu of them) land and issued MMAs are done.  (Otherwise the last pass's accumulators, which every
+    // copy and MMA precedes, have been read.)
+    if (!__syncthreads_and(ok ? 1 : 0)) {
+        if (warp == NGW && lane == 0)
+            for (int g = max(0, gu - SM::NBUF); g < gu; ++g) umma::mbar_wait_sleep(umma::smem_u32(&bfull[g % SM::NBUF]), (g / SM::NBUF) & 1);
+        if (warp > NGW && lane == 0) {
+            commit(&mdone[warp - NGW - 1]);
+            umma::mbar_wait_sleep(umma::smem_u32(&mdone[warp - NGW - 1]), 0);
+        }
+    }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");

@@ -249,6 +249,7 @@ struct EvalArgs {
     const longlong2 *trig;  // e^{2 pi i j/GF_TRIG_STEPS}, 2^61 for 1
     const int *rej;
     int *err;               // device error word of the plan (bounded waits)
+    int drop_unit, drop_warp; // self-test of the products' waits: drop_unit - 1 (0: none) of warp drop_warp (farmma.cu)
 };
 
 #define GF_TRIG_STEPS 1024

@@ -774,12 +774,14 @@ static int64_t far_segment_size(int64_t n)
     return segs <= 1024 ? 512 : ((n + 1023) / 1024 + 31) / 32 * 32;
 }
 
-gf_status gf_eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int which, void *dev_out,
-                         void *cuda_stream)
+static gf_status eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int which, void *dev_out, int drop_warp, int drop_unit,
+                             void *cuda_stream)
 {
     EvalArgs a;
     gf_status s = gf_plan_eval_args(p, dev_xyz, n, which, dev_out, &a, "gf_eval_points");
     if (s != GF_OK || n == 0) return s;
+    a.drop_warp = drop_warp;
+    a.drop_unit = drop_unit;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     // per-call scratch from the stream-ordered pool on the caller's stream, returned
     // to the pool in stream order after the kernels: concurrent calls on other
@@ -842,6 +844,24 @@ gf_status gf_eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int whic
     gf_dev_free(scratch, st);
     CU(e);
     return GF_OK;
+}
+
+gf_status gf_eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int which, void *dev_out, void *cuda_stream)
+{
+    return eval_points(p, dev_xyz, n, which, dev_out, 0, 0, cuda_stream);
+}
+
+gf_status gf_eval_wait_selftest(gf_plan_t p, const double *dev_xyz, int64_t n, int which, void *dev_out, int warp, int unit,
+                                void *cuda_stream)
+{
+    if (!p || warp < 0 || warp > 4 || unit < -1) return fail(GF_ERR_ARG, "gf_eval_wait_selftest: bad argument");
+    gf_status s = gf_plan_status(p, cuda_stream);
+    if (s != GF_OK) return fail(GF_ERR_ARG, "gf_eval_wait_selftest: the plan's error word is set already");
+    if ((s = eval_points(p, dev_xyz, n, which, dev_out, warp, unit + 1, cuda_stream)) != GF_OK) return s;
+    if (gf_plan_status(p, cuda_stream) == GF_OK) return GF_OK;
+    CU(cudaMemsetAsync(p->errw, 0, sizeof(int), (cudaStream_t)cuda_stream));
+    CU(cudaStreamSynchronize((cudaStream_t)cuda_stream));
+    return fail(GF_ERR_TIMEOUT, "gf_eval_wait_selftest: the bounded wait ran out");
 }
 
 }  // extern "C"
