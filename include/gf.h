@@ -390,11 +390,14 @@ gf_status gf_surrogate_eval_residual(gf_mlp_t mlp, int npairs, const double *k, 
                                      int *n_fallback_pairs, void *cuda_stream);
 gf_status gf_mlp_destroy(gf_mlp_t mlp);
 
-/* Device status of a plan's synthesis: the inverse-FFT passes stage their tiles
- * with TMA copies completed on mbarriers, and every such wait has a poll limit;
- * a wait that ran out sets the plan's device error word instead of hanging.
- * Synchronises cuda_stream, then returns GF_ERR_TIMEOUT if the word is set,
- * GF_OK otherwise.  Errors: GF_ERR_ARG, GF_ERR_CUDA. */
+/* Device status of a plan: the synthesis' last pass stages its rows, and the matrix
+ * products of long evaluations (gf_eval_points, gf_eval_points_host) their operands, by
+ * copies completed on mbarriers.  Every such wait is bounded; one that ran out sets the
+ * plan's device error word instead of hanging.  The call it belongs to has returned
+ * GF_OK (its work was only queued): a grid, or the outputs of the evaluations since the last
+ * check, are then not to be used.  The word stays set.  Synchronises cuda_stream,
+ * then returns GF_ERR_TIMEOUT if the word is set, GF_OK otherwise.  Errors:
+ * GF_ERR_ARG, GF_ERR_CUDA. */
 gf_status gf_plan_status(gf_plan_t plan, void *cuda_stream);
 
 /* Self-test of the bounded waits of the far series' matrix products (diagnostic):

@@ -116,7 +116,7 @@ struct gf_plan_s {
     // far-region grid (far_grid_M > 0): [fNZ][fM + 3][fM + 3][nf], plane m at z = fz0 + m fhz
     void *fargrid = nullptr;
     size_t far_bytes = 0;
-    int *errw = nullptr;              // device error word of the synthesis (bounded waits)
+    int *errw = nullptr;              // device error word of synthesis and evaluations (bounded waits)
     int fM = 0, fNZ = 0;
     double fz0 = 0, fhz = 0, fzmax = 0;
     size_t elem = 16;                 // bytes per complex value
@@ -1073,7 +1073,7 @@ gf_status gf_plan_status(gf_plan_t p, void *cuda_stream)
     cudaStream_t st = (cudaStream_t)cuda_stream;
     CU(cudaMemcpyAsync(&host, p->errw, sizeof(int), cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
-    if (host) return fail(GF_ERR_TIMEOUT, "gf_plan_status: a bounded wait for staged copies ran out in the synthesis");
+    if (host) return fail(GF_ERR_TIMEOUT, "gf_plan_status: a bounded wait ran out in the plan's synthesis or in an evaluation");
     return GF_OK;
 }
 

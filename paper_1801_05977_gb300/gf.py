@@ -293,7 +293,8 @@ class Plan:
                                                ctypes.c_void_p(out.data_ptr()), int(warp), int(unit), _stream_ptr(stream)))
 
     def status(self, stream=None) -> int:
-        """gf_plan_status: GF_OK, or GF_ERR_TIMEOUT if a bounded wait of the synthesis ran out."""
+        """gf_plan_status: GF_OK, or GF_ERR_TIMEOUT if a bounded wait of the synthesis or of an evaluation
+        ran out."""
         return int(lib().gf_plan_status(self._h, _stream_ptr(stream)))
 
     def phase_ms(self):
