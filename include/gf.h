@@ -338,7 +338,9 @@ gf_status gf_mlp_params(gf_mlp_t mlp, float *host, int64_t count, int to_device)
 /* Scale of the targets: the network learns L_d / scale. */
 gf_status gf_mlp_set_scale(gf_mlp_t mlp, double scale);
 /* Forward pass of n samples (device pointers), output float [n][2]: one fused
- * persistent tensor-core kernel (activations stay on chip). */
+ * persistent tensor-core kernel (activations stay on chip).  The output may lie over
+ * the input (which is copied first, into the network's own buffer: such calls on one
+ * network must not overlap in time). */
 gf_status gf_mlp_forward(gf_mlp_t mlp, const float *dev_in, int n, float *dev_out, void *cuda_stream);
 /* One Adam step (lr; beta 0.9/0.999) on the mean-squared loss
  * sum (Y - T)^2 / (2n) of one batch (targets float [n][2]); the batch loss is
