@@ -180,13 +180,16 @@ size_t gf_grid_bytes(gf_plan_t plan);
  * The plan is not modified by an evaluation: each call takes its scratch (the
  * far- and near-branch target lists, 12 bytes per target plus 9 KiB; for 3D
  * plans also about 8 bytes per target (4 MiB at most) of far-list counts and
- * tickets, the far sums' slab partials, 4 * entries * (8 or 16) bytes per target
- * for float or double plans (up to 16 times that below 16384 targets), and, from
- * 12288 to 327680 targets on (by precision and kind), the far weights' images:
+ * tickets, the far sums' slab partials, entries * (8 or 16) bytes (float or double
+ * plans) times 64 per target up to 16384 targets, then 2^20 up to 262144 and 4 per
+ * target beyond, and, from 12288 (double Helmholtz), 20480 (double Maxwell), 327680
+ * (split Maxwell) or 786432 targets (split Helmholtz) on, the far weights' images:
  * 61 MB (double) or 10 MB (float) per entry) from the library's stream-ordered
  * memory pool on cuda_stream
  * and returns it in stream order, so calls on one plan may run concurrently on
- * different streams and threads.  Results are reproducible: the same plan and
+ * different streams and threads.  Where that much memory is not to be had the call
+ * does with 4 slab slots per target and no images (the far sums then go another way and
+ * differ in their roundings).  Otherwise results are reproducible: the same plan and
  * targets give the same bits at every call (the far targets are grouped by a
  * stable sort, and each far sum adds its row-slab partials in slab order).
  * For 3D double-precision Helmholtz plans

@@ -788,20 +788,31 @@ static gf_status eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int 
     // streams each have their own, and the plan stays unchanged
     const bool slabs = p->dim == 3;
     // slab partials: two slots per target, up to 32 for short lists (they use more slabs)
-    const int64_t npad = (n + 31) / 32 * 32, nchmax = npad / 32, slabcap = npad <= (1 << 14) ? 32 * npad : std::max<int64_t>(2 * npad, 1 << 19);
+    const int64_t npad = (n + 31) / 32 * 32, nchmax = npad / 32;
+    int64_t slabcap = npad <= (1 << 14) ? 32 * npad : std::max<int64_t>(2 * npad, 1 << 19);
     const int64_t segsize = far_segment_size(n), nseg = (n + segsize - 1) / segsize;
     const size_t ints = (size_t)(GF_COUNTER_PAD + 3 * n + (slabs ? 2 * nchmax + nseg * GF_FAR_BUCKETS : 0));
     const size_t off_buf = (sizeof(int) * ints + 255) / 256 * 256;
-    const size_t buf_bytes = slabs ? (size_t)slabcap * gf_out_entries(which) * p->elem : 0;
+    size_t buf_bytes = slabs ? (size_t)slabcap * gf_out_entries(which) * p->elem : 0;
     // far targets by matrix products: from gf_far_product_min targets on, propagating indices
     // within the one block of rows that the products give them (k < 7), no far-region grid
     size_t mma_bytes = 0;
     int mma_cells = 0;
     if (slabs && n >= gf_far_product_min(p->precision, p->nf) && p->k < 7.0 && !p->fargrid && which != GF_OUT_LD)
         mma_bytes = gf_far_product_bytes(p->precision, n, p->nf == 1 ? 1 : gf_out_entries(which), &mma_cells);
-    const size_t off_mma = (off_buf + 2 * buf_bytes + 255) / 256 * 256;
+    size_t off_mma = (off_buf + 2 * buf_bytes + 255) / 256 * 256;
     int *scratch = nullptr;
-    CU(gf_dev_alloc((void **)&scratch, off_mma + mma_bytes, st));
+    cudaError_t e = gf_dev_alloc((void **)&scratch, off_mma + mma_bytes, st);
+    if (e == cudaErrorMemoryAllocation && slabs && (mma_bytes || slabcap > 2 * npad)) {
+        // what the series kernels need at least: no images, two slab slots per target
+        cudaGetLastError();
+        mma_bytes = 0;
+        slabcap = 2 * npad;
+        buf_bytes = (size_t)slabcap * gf_out_entries(which) * p->elem;
+        off_mma = (off_buf + 2 * buf_bytes + 255) / 256 * 256;
+        e = gf_dev_alloc((void **)&scratch, off_mma, st);
+    }
+    CU(e);
     if (mma_bytes) {
         a.mma = (char *)scratch + off_mma;
         a.mma_cells = mma_cells;
@@ -810,7 +821,7 @@ static gf_status eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int 
     a.far_idx = scratch + GF_COUNTER_PAD;
     a.far_sorted = a.far_idx + n;
     a.near_idx = p->dim == 3 ? a.far_idx + 2 * n : nullptr;
-    cudaError_t e = cudaMemsetAsync(a.far_count, 0, sizeof(int) * GF_SCRATCH_COUNTERS, st);
+    e = cudaMemsetAsync(a.far_count, 0, sizeof(int) * GF_SCRATCH_COUNTERS, st);
     if (slabs && e == cudaSuccess) {
         a.slabtick[0] = a.far_idx + 3 * n;
         a.slabtick[1] = a.slabtick[0] + nchmax;
