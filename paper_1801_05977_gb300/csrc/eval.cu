@@ -2365,73 +2365,24 @@ __device__ __forceinline__ int far_take(int *counter, int nitems)
 // The float sums' set-up is cheap, their rows short: half as many.
 constexpr int FAR_SLABS_SHORT = 64, FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_SHORT = 24, FAR_LONG = 300;
 
-// Chunks of a far launch: all of the list, or those of the cells that the product
-// path left over (a.rej: their number, tiles per cell, a flag per cell).  The t-th
-// chunk taken from the end of the list is `at(t)`, -1 where the last cell ends
-// short of its tiles.  Called by all threads of the block.
-struct FarChunks {
-    int nch, count, per;
-    const short *cell;
-    __device__ __forceinline__ FarChunks(const EvalArgs &a, short *list)
-    {
-        count = a.far_count[0];
-        nch = (count + 31) >> 5;
-        per = 0;
-        cell = nullptr;
-        if (a.rej) {
-            per = 4 * a.rej[1];
-            const int nrej = a.rej[0], ncell = (nch + per - 1) / per;
-            if (nrej > 0) {
-                // the flagged cells in order, by one warp
-                if (threadIdx.x < 32) {
-                    int n = 0;
-                    for (int c0 = 0; c0 < ncell; c0 += 32) {
-                        const int c = c0 + (int)threadIdx.x;
-                        const bool f = c < ncell && a.rej[2 + c] != 0;
-                        const unsigned bal = __ballot_sync(0xffffffffu, f);
-                        if (f) list[n + __popc(bal & ((1u << threadIdx.x) - 1u))] = (short)c;
-                        n += __popc(bal);
-                    }
-                }
-                __syncthreads();
-            }
-            nch = nrej * per;
-            cell = list;
-        }
-    }
-    __device__ __forceinline__ int at(int t) const
-    {
-        const int w = nch - 1 - t;
-        if (!cell) return w;
-        const int c = cell[w / per] * per + w % per;
-        return c * 32 < count ? c : -1;
-    }
-    // row slabs per chunk: by the chunks of this launch, capped by the scratch of the whole list
-    __device__ __forceinline__ int slabs(const EvalArgs &a, int kind, bool fp64) const
-    {
-        const int s = nch <= FAR_SHORT ? FAR_SLABS_SHORT : nch <= FAR_LONG || !fp64 ? FAR_SLABS_MAX : FAR_SLABS_LONG;
-        const int smax = fp64 ? s : s / 2;
-        return far_slabs_capped(a, kind, (count + 31) >> 5, far_slabs(nch, smax));
-    }
-    // the same for items of two chunks
-    __device__ __forceinline__ int slabs2(const EvalArgs &a, int items) const
-    {
-        return far_slabs_capped(a, 0, (count + 31) >> 5, far_slabs(items, FAR_SLABS_MAX / 2, 2));
-    }
-};
-static_assert(GF_FAR_CELLS < 32768, "cells are listed as short");
+// Row slabs per chunk of a far launch over `count` targets (a.nfar: the far list, or what the
+// products left of it, a list of its own: a look-up of the left chunks in the kernels cost far3d_f64 registers
+// and shared memory that kept the tails from running beside it, a million targets with k = 7.3 7.65 -> 8.95 ms,
+// |x3| <= 3 4.70 -> 8.80).
+__device__ __forceinline__ int far_chunk_slabs(const EvalArgs &a, int kind, bool fp64, int nch)
+{
+    const int s = nch <= FAR_SHORT ? FAR_SLABS_SHORT : nch <= FAR_LONG || !fp64 ? FAR_SLABS_MAX : FAR_SLABS_LONG;
+    return far_slabs_capped(a, kind, nch, far_slabs(nch, fp64 ? s : s / 2));
+}
 
 template <int NF, bool TAILS>
 __global__ void __launch_bounds__(128, NF == 1 ? 5 : 1) far3d_f64(EvalArgs a)
 {
-    __shared__ short rejected[GF_FAR_CELLS];
-    const FarChunks ch(a, rejected);
-    const int S = ch.slabs(a, 0, true);
+    const int count = *a.nfar;
+    const int nch = (count + 31) >> 5, S = far_chunk_slabs(a, 0, true, nch);
     int *ctr = a.far_count + GF_WORK_SLOT;
-    for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
-        const int w = ch.at(t / S);
-        if (w >= 0) far3d_f64_chunk<NF, TAILS>(a, w, ch.count, t % S, S);
-    }
+    for (int t = far_take(ctr, nch * S); t >= 0; t = far_take(ctr, nch * S))
+        far3d_f64_chunk<NF, TAILS>(a, nch - 1 - t / S, count, t % S, S);
 }
 
 // ---------------------------------------------------------------------------
@@ -2524,14 +2475,11 @@ __device__ void far3d_tail_chunk(const EvalArgs &a, int w, int count, int slab, 
 template <int NF>
 __global__ void __launch_bounds__(128) far3d_tail(EvalArgs a)
 {
-    __shared__ short rejected[GF_FAR_CELLS];
-    const FarChunks ch(a, rejected);
-    const int S = ch.slabs(a, 1, true);
+    const int count = *a.nfar;
+    const int nch = (count + 31) >> 5, S = far_chunk_slabs(a, 1, true, nch);
     int *ctr = a.far_count + GF_TAIL_SLOT;
-    for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
-        const int w = ch.at(t / S);
-        if (w >= 0) far3d_tail_chunk<NF>(a, w, ch.count, t % S, S);
-    }
+    for (int t = far_take(ctr, nch * S); t >= 0; t = far_take(ctr, nch * S))
+        far3d_tail_chunk<NF>(a, nch - 1 - t / S, count, t % S, S);
 }
 
 // ---------------------------------------------------------------------------
@@ -2880,25 +2828,23 @@ constexpr int FAR_PAIRS = 1;
 template <int NF>
 __global__ void __launch_bounds__(128, NF == 1 ? 6 : 1) far3d_f32(const __grid_constant__ EvalArgs a)
 {
-    __shared__ short rejected[GF_FAR_CELLS];
-    const FarChunks ch(a, rejected);
+    const int count = *a.nfar, nch = (count + 31) >> 5;
     int *ctr = a.far_count + GF_WORK_SLOT;
-    if (NF == 1 && ch.nch >= FAR_PAIRS * (int)(gridDim.x * blockDim.x >> 5)) {
-        const int np = (ch.nch + 1) >> 1, S = ch.slabs2(a, np);
+    if (NF == 1 && nch >= FAR_PAIRS * (int)(gridDim.x * blockDim.x >> 5)) {
+        const int np = (nch + 1) >> 1, S = far_slabs_capped(a, 0, nch, far_slabs(np, FAR_SLABS_MAX / 2, 2));
         for (int t = far_take(ctr, np * S); t >= 0; t = far_take(ctr, np * S)) {
             const int u = 2 * (t / S);
-            far3d_f32_helm<2>(a, {ch.at(u), u + 1 < ch.nch ? ch.at(u + 1) : -1}, ch.count, t % S, S);
+            far3d_f32_helm<2>(a, {nch - 1 - u, nch - 2 - u}, count, t % S, S);
         }
         return;
     }
-    const int S = ch.slabs(a, 0, false);
-    for (int t = far_take(ctr, ch.nch * S); t >= 0; t = far_take(ctr, ch.nch * S)) {
-        const int w = ch.at(t / S);
-        if constexpr (NF > 1) {
-            if (w >= 0) far3d_f32_maxwell(a, w, ch.count, t % S, S);
-        } else if (w >= 0) {
-            far3d_f32_helm<1>(a, {w}, ch.count, t % S, S);
-        }
+    const int S = far_chunk_slabs(a, 0, false, nch);
+    for (int t = far_take(ctr, nch * S); t >= 0; t = far_take(ctr, nch * S)) {
+        const int w = nch - 1 - t / S;
+        if constexpr (NF > 1)
+            far3d_f32_maxwell(a, w, count, t % S, S);
+        else
+            far3d_f32_helm<1>(a, {w}, count, t % S, S);
     }
 }
 
@@ -3311,6 +3257,7 @@ template <typename R>
 cudaError_t launch_eval_t(const EvalArgs &a0, cudaStream_t s, cudaEvent_t ev_mid, const EvalFork *fork)
 {
     EvalArgs a = a0;
+    a.nfar = a.far_count;
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

@@ -122,7 +122,7 @@ __device__ float digit_radius(float z, int p, int i, float ldelta, float lfact, 
 // One block per cell: the |x3| range of its targets, the expansion's orders, the
 // rows of every digit and the layout of its images.  Cells that the product kernel
 // cannot take (too wide in |x3|, too many rows, columns or bytes) are flagged for the
-// series kernels: rej[0] their number, rej[1] tiles per cell, rej[2 + cell] 1.
+// series kernels: rej[0] the number of their targets, rej[1] tiles per cell, rej[2 + cell] 1.
 template <int L>
 __global__ void __launch_bounds__(128) far_cells(EvalArgs a, Cell *cells, int *rej, int maxcells, int out_e)
 {
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(128) far_cells(EvalArgs a, Cell *cells, int *r
     C.npu = npu;
     C.ok = ok ? 1 : 0;
     rej[2 + c] = ok ? 0 : 1;
-    if (!ok) atomicAdd(rej, 1);
+    if (!ok) atomicAdd(rej, s1 - s0);
     cells[c] = C;
 }
 
@@ -509,7 +509,7 @@ __device__ __forceinline__ uint32_t pair_at(int i, long long a, long long b)
 __device__ __forceinline__ long long recip61(int p) { return (1ll << 61) / p; }
 
 template <int L>
-__global__ void __launch_bounds__(256) far_weights(EvalArgs a, const Cell *cells, const int *rej, unsigned char *images, int maxcells, int nent)
+__global__ void __launch_bounds__(256) far_weights(EvalArgs a, const Cell *cells, int *rej, unsigned char *images, int maxcells, int nent)
 {
     __shared__ Cell C;
     __shared__ long long rcp[PMAX + 1];
@@ -522,7 +522,16 @@ __global__ void __launch_bounds__(256) far_weights(EvalArgs a, const Cell *cells
     }
     if (threadIdx.x >= 1 && threadIdx.x <= PMAX) rcp[threadIdx.x] = recip61(threadIdx.x);
     __syncthreads();
-    if (!C.ok) return;
+    if (!C.ok) {
+        // left over: its targets go to the series kernels' list, after those of the flagged cells before it (only the
+        // last cell is shorter than T tiles, so the list's chunks are the far list's)
+        if (kb != NKB) return;
+        static_assert(GF_FAR_CELLS <= 256, "a thread per cell");
+        const int before = __syncthreads_count(threadIdx.x < c && rej[2 + threadIdx.x] != 0);
+        const int per = T * TILE, count = a.far_count[0];
+        for (int i = threadIdx.x; i < per && c * per + i < count; i += blockDim.x) rej[2 + maxcells + before * per + i] = a.far_sorted[c * per + i];
+        return;
+    }
     if (kb == NKB && C.merged) return;
     const int kcol = kb == NKB ? 0 : kb;
     const int N1 = (int)rint(-a.a1), N2 = (int)rint(-a.a2);
@@ -1451,7 +1460,10 @@ __global__ void __launch_bounds__(THREADS, 1) far_product(EvalArgs a, const Cell
 
 }  // namespace
 
-// Bytes of scratch for n targets (cells, list of cells left over, images) and the
+// Cells' flags and the targets left over (at most all), before the images.
+static size_t rej_bytes(int nc, int64_t n) { return (sizeof(int) * (nc + 2 + n) + 255) / 256 * 256; }
+
+// Bytes of scratch for n targets (cells, list of targets left over, images) and the
 // number of cells; 0 bytes: no product path for so few targets.
 size_t gf_far_product_bytes(int precision, int64_t n, int nent, int *maxcells)
 {
@@ -1459,7 +1471,7 @@ size_t gf_far_product_bytes(int precision, int64_t n, int nent, int *maxcells)
     const int nc = (int)(tiles < GF_FAR_CELLS ? tiles : GF_FAR_CELLS);
     *maxcells = nc;
     const size_t img = precision == GF_FP64 ? (size_t)Cap<6>::BYTES : (size_t)Cap<3>::BYTES;
-    return (sizeof(Cell) * nc + 255) / 256 * 256 + (sizeof(int) * (nc + 2) + 255) / 256 * 256 + img * nc * nent;
+    return (sizeof(Cell) * nc + 255) / 256 * 256 + rej_bytes(nc, n) + img * nc * nent;
 }
 
 template <typename R, int L>
@@ -1469,7 +1481,7 @@ static cudaError_t launch_product(EvalArgs &a, int nsm, cudaStream_t s)
     unsigned char *p = reinterpret_cast<unsigned char *>(a.mma);
     Cell *cells = reinterpret_cast<Cell *>(p);
     int *rej = reinterpret_cast<int *>(p + (sizeof(Cell) * nc + 255) / 256 * 256);
-    unsigned char *img = reinterpret_cast<unsigned char *>(rej) + (sizeof(int) * (nc + 2) + 255) / 256 * 256;
+    unsigned char *img = reinterpret_cast<unsigned char *>(rej) + rej_bytes(nc, a.n);
     cudaError_t e = cudaFuncSetAttribute(far_product<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<L>::TOTAL);
     if (e != cudaSuccess) return e;
     const int ne = a.nf == 1 ? 1 : gf_out_entries(a.which);
@@ -1478,12 +1490,13 @@ static cudaError_t launch_product(EvalArgs &a, int nsm, cudaStream_t s)
     far_weights<L><<<dim3(nc, NKB + 1), 256, 0, s>>>(a, cells, rej, img, nc, ne);
     far_product<R, L><<<nsm, THREADS, Smem<L>::TOTAL, s>>>(a, cells, rej, img, nc, ne, a.err);
     gf_count_launch(3);
-    a.rej = rej;
+    a.nfar = rej;
+    a.far_sorted = rej + 2 + nc;
     return cudaGetLastError();
 }
 
-// The far targets' series by matrix products; cells it leaves over are listed in
-// a.rej for the series kernels.
+// The far targets' series by matrix products; a.far_sorted and a.nfar are then the list of
+// those left to the series kernels.
 cudaError_t gf_launch_far_product(EvalArgs &a, int precision, int nsm, cudaStream_t s)
 {
     unsigned char *p = reinterpret_cast<unsigned char *>(a.mma);

@@ -242,12 +242,11 @@ struct EvalArgs {
     double bmin;            // smallest |beta_n| over the evanescent n (this value or a larger one, never smaller)
     double bprop;           // smallest beta_n over the propagating n (0: there are none)
     // far series by matrix products (3D; null: by the series kernels alone): scratch of
-    // mma_cells cells; rej: cells left to the series kernels (their number, 128-target
-    // tiles per cell, the cells), null: every far target is theirs
+    // mma_cells cells
     void *mma;
     int mma_cells;
     const longlong2 *trig;  // e^{2 pi i j/GF_TRIG_STEPS}, 2^61 for 1
-    const int *rej;
+    const int *nfar;        // number of entries of far_sorted that the series kernels sum (single evaluations)
     int *err;               // device error word of the plan (bounded waits)
     int drop_unit, drop_warp; // self-test of the products' waits: drop_unit - 1 (0: none) of warp drop_warp (farmma.cu)
 };
