@@ -183,7 +183,8 @@ size_t gf_grid_bytes(gf_plan_t plan);
  * tickets, the far sums' slab partials, entries * (8 or 16) bytes (float or double
  * plans) times 64 per target up to 16384 targets, then 2^20 up to 262144 and 4 per
  * target beyond, and, from 12288 (double Helmholtz), 20480 (double Maxwell), 327680
- * (split Maxwell) or 786432 targets (split Helmholtz) on, 4 bytes per target and the far weights' images:
+ * (split Maxwell) or 786432 targets (split Helmholtz) on (times (c/0.6)^1.4 for c
+ * above 0.6), 4 bytes per target and the far weights' images:
  * 61 MB (double) or 10 MB (float) per entry) from the library's stream-ordered
  * memory pool on cuda_stream
  * and returns it in stream order, so calls on one plan may run concurrently on

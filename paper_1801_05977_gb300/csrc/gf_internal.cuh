@@ -257,14 +257,17 @@ struct EvalArgs {
 #ifndef GF_FAR_CELLS
 #define GF_FAR_CELLS 152
 #endif
-// Targets from which an evaluation takes the product path (uniform targets, |x3| <= 1, times of
-// the whole evaluation, series kernels against products): double Helmholtz 263 / 418 us at 8000
-// (there the cells are too wide in |x3|), 408 / 286 at 16000; double Maxwell 1090 / 1312 at 16000,
-// 1832 / 967 at 32000; split Helmholtz 356 / 363 at 512000, 556 / 541 at a million (k = 5: 381 / 374, 608 / 555);
-// split Maxwell 704 / 714 at 256000, 1264 / 1150 at 512000.
-inline int64_t gf_far_product_min(int precision, int nf)
+// Targets from which an evaluation takes the product path (uniform targets, |x3| <= 1, c = 0.6, times of
+// the whole evaluation, series kernels against products): double Helmholtz 260 / 294 us at 12500, 365 / 294 at 25000;
+// double Maxwell 911 / 897 at 12500, 1622 / 1231 at 25000; split Helmholtz 462 / 463 at 800000; split Maxwell 553 / 553 at
+// 200000, 905 / 821 at 400000.  A far target's series has about (T/c)^2 terms at most, the products' cost hardly
+// depends on it: with c = 1.2 they meet at 40000 (double Helmholtz; 388 / 306 at 100000) and 45000 targets (double
+// Maxwell), with c = 2 at 60000 and 100000, with c = 3 at 140000 (518 / 357 at 200000) and 180000; with c = 0.8 split
+// Maxwell 620 / 665 at 400000.
+inline int64_t gf_far_product_min(int precision, int nf, double c)
 {
-    return precision == GF_FP64 ? (nf == 1 ? 12288 : 20480) : (nf == 1 ? 786432 : 327680);
+    const double n = precision == GF_FP64 ? (nf == 1 ? 12288 : 20480) : (nf == 1 ? 786432 : 327680);
+    return c > 0.6 ? (int64_t)fmin(n * pow(c / 0.6, 1.4), 1e18) : (int64_t)n;
 }
 size_t gf_far_product_bytes(int precision, int64_t n, int nent, int *maxcells);
 cudaError_t gf_launch_far_product(EvalArgs &a, int precision, int nsm, cudaStream_t s);

@@ -798,7 +798,7 @@ static gf_status eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int 
     // within the one block of rows that the products give them (k < 7), no far-region grid
     size_t mma_bytes = 0;
     int mma_cells = 0;
-    if (slabs && n >= gf_far_product_min(p->precision, p->nf) && p->k < 7.0 && !p->fargrid && which != GF_OUT_LD)
+    if (slabs && n >= gf_far_product_min(p->precision, p->nf, p->tr.c) && p->k < 7.0 && !p->fargrid && which != GF_OUT_LD)
         mma_bytes = gf_far_product_bytes(p->precision, n, p->nf == 1 ? 1 : gf_out_entries(which), &mma_cells);
     size_t off_mma = (off_buf + 2 * buf_bytes + 255) / 256 * 256;
     int *scratch = nullptr;
