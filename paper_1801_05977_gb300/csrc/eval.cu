@@ -2362,8 +2362,10 @@ __device__ __forceinline__ int far_take(int *counter, int nitems)
 // 300 chunks on the slabs' repeated set-up costs more (13000 far targets: 559 us for
 // the evaluation with 8 slabs, 681 us with 32).  Up to some 24 chunks even single rows pay (whole
 // evaluations with 32 / 64 / 128 slabs: 1017 targets 146 / 132 / 131 us, 3000 targets 153 / 159 / 177).
-// The float sums' set-up is cheap, their rows short: half as many.
-constexpr int FAR_SLABS_SHORT = 64, FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_SHORT = 24, FAR_LONG = 300;
+// The float sums' set-up is cheap, their rows short: half as many.  These figures are for c = 0.6, 133 rows a
+// target.  With fewer rows (larger c) a slab has two of them at least and a list is long sooner (25000 targets, a quarter
+// of them far: c = 3, 27 rows 226 us with 32 slabs, 171 with 8; c = 1.2, 67 rows 246 and 190).
+constexpr int FAR_SLABS_SHORT = 64, FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_SHORT = 24, FAR_LONG = 300, FAR_HALF_ROWS = 66;
 
 // Row slabs per chunk of a far launch over `count` targets (a.nfar: the far list, or what the
 // products left of it, a list of its own: a look-up of the left chunks in the kernels cost far3d_f64 registers
@@ -2371,8 +2373,11 @@ constexpr int FAR_SLABS_SHORT = 64, FAR_SLABS_MAX = 32, FAR_SLABS_LONG = 8, FAR_
 // |x3| <= 3 4.70 -> 8.80).
 __device__ __forceinline__ int far_chunk_slabs(const EvalArgs &a, int kind, bool fp64, int nch)
 {
-    const int s = nch <= FAR_SHORT ? FAR_SLABS_SHORT : nch <= FAR_LONG || !fp64 ? FAR_SLABS_MAX : FAR_SLABS_LONG;
-    return far_slabs_capped(a, kind, nch, far_slabs(nch, fp64 ? s : s / 2));
+    const float Tc = (float)a.T / (float)a.c, kf = (float)a.k;
+    const int half_rows = (int)fminf(sqrtf(fmaf(Tc, Tc, kf * kf)), 1e6f);  // at |x3| = c
+    const int longer = FAR_LONG * min(half_rows, FAR_HALF_ROWS) / FAR_HALF_ROWS;
+    const int s = nch <= FAR_SHORT ? FAR_SLABS_SHORT : nch <= longer || !fp64 ? FAR_SLABS_MAX : FAR_SLABS_LONG;
+    return far_slabs_capped(a, kind, nch, far_slabs(nch, max(FAR_SLABS_LONG, min(fp64 ? s : s / 2, half_rows))));
 }
 
 template <int NF, bool TAILS>
