@@ -3146,7 +3146,7 @@ __global__ void __launch_bounds__(F2_THR) far2d(const __grid_constant__ EvalArgs
                 acc[e][0] += __shfl_xor_sync(0xffffffffu, acc[e][0], o);
                 acc[e][1] += __shfl_xor_sync(0xffffffffu, acc[e][1], o);
             }
-        if (sub == 0 && slot < count) {
+        if (sub == 0 && slot < nt) {
             const double2 lat = lattice_phase(a.a1, m, 0.0, 0.0);
             const double2 pre = cmul(lat, make_double2(0.0, 0.25 / GF_PI));
             for (int e = 0; e < ne; ++e)
