@@ -2924,6 +2924,10 @@ constexpr int F2_THR = 512;
 constexpr int F2_TAB = 1024;            // indices kept (the middle of the range)
 constexpr int F2_Y = 48;                // the exponential's table, y < F2_Y
 constexpr int F2_S = 64;                // steps per unit of y
+// Indices of a lane's run to either side of the middle at |x2| = c: with a small c the targets nearest the slab have
+// thousands, and a warp of them would outlast all others (c = 0.01, 4000 indices, 50,000 targets with |x2| <= 0.3: 11.1 ms with
+// a lane a target).  Default plans have 67.
+constexpr int F2_RUN = 512;
 
 // (|beta_n|, 1/|beta_n|), the first negative for a propagating n.
 __device__ __forceinline__ double2 ei_beta(double kk, double c1)
@@ -2951,7 +2955,7 @@ __device__ __forceinline__ double exp_neg_tab(double y, const double *T)
 }
 
 template <typename R, int OUT>
-__global__ void __launch_bounds__(F2_THR) far2d(const __grid_constant__ EvalArgs a)
+__global__ void __launch_bounds__(F2_THR) far2d(const __grid_constant__ EvalArgs a, int lgmin)
 {
     typedef typename cplx_t<R>::T C;
     constexpr bool hess = OUT == GF_OUT_HESSDIFF, grad = OUT == GF_OUT_GRAD;
@@ -2990,7 +2994,7 @@ __global__ void __launch_bounds__(F2_THR) far2d(const __grid_constant__ EvalArgs
     }
     // the CTA's share of the targets; lanes per target
     const int share = (count + gridDim.x - 1) / gridDim.x, c0 = blockIdx.x * share, c1e = min(count, c0 + share);
-    int lgl = 0;
+    int lgl = lgmin;
     while (lgl < 5 && (share << (lgl + 1)) <= 128) ++lgl;
     const int lpt = 1 << lgl, sub = threadIdx.x & (lpt - 1), chunk = F2_THR >> lgl;
     for (int base = c0; base < c1e; base += chunk) {
@@ -3155,13 +3159,26 @@ __global__ void __launch_bounds__(F2_THR) far2d(const __grid_constant__ EvalArgs
     }
 }
 
-// Short lists: a warp per target, lanes over the indices, every term by itself.  No tables to fill and no
+// Lists by a warp per target, lanes over the indices, every term by itself.  Short lists: no tables to fill and no
 // order to make, which is most of far2d's time there: whole evaluations of 1 / 1000 / 3000 targets (40% far) G 48 / 70 / 95
 // us against far2d's 59 / 81 / 99, GRAD 50 / 80 / 108 against 64 / 91 / 110, HESSDIFF 59 / 92 / 137 against 66 / 97 / 131.
+// And lists whose targets near |x2| = c have more indices R than far2d's table, up to 16 R targets or where most of the
+// indices propagate (far2d passes them twice): 50,000 targets |x2| <= 0.3, c = 0.01 (R = 4000) 5.6 ms against 6.8, c = 0.002 9.6
+// against 14.7, c = 0.03 3.7 against 3.2; |x2| <= 1, c = 0.6, k = 900 4.4 against 6.1, k = 300 1.74 against 1.53.
 constexpr int64_t F2_SHORT = 2048;      // targets
 
+// -1: by a warp per target; else far2d's least number of lanes a target (its logarithm).
+inline int far2d_route(const EvalArgs &a)
+{
+    const double kmax = a.which == GF_OUT_HESSDIFF ? fmax(a.k, a.k2) : a.k, Tc = a.T / a.c, R = sqrt(kmax * kmax + Tc * Tc);
+    if (a.n <= F2_SHORT || (R > F2_TAB / 2 - 5 && ((double)a.n <= 16.0 * R || kmax > F2_TAB / 2 - 5))) return -1;
+    int lg = 0;
+    while (lg < 5 && R > (double)(F2_RUN << std::max(lg - 1, 0))) ++lg;
+    return lg;
+}
+
 template <typename R, int OUT>
-__global__ void __launch_bounds__(128) far2d_short(const __grid_constant__ EvalArgs a)
+__global__ void __launch_bounds__(128) far2d_warps(const __grid_constant__ EvalArgs a)
 {
     typedef typename cplx_t<R>::T C;
     constexpr int ne = OUT == GF_OUT_G ? 1 : 3;
@@ -3235,14 +3252,15 @@ __global__ void __launch_bounds__(128) far2d_short(const __grid_constant__ EvalA
 template <typename R, int OUT>
 cudaError_t launch_far2d(const EvalArgs &a, int nsm, cudaStream_t s)
 {
-    if (a.n <= F2_SHORT) {
-        far2d_short<R, OUT><<<(int)((a.n + 3) / 4), 128, 0, s>>>(a);
+    const int lgmin = far2d_route(a);
+    if (lgmin < 0) {
+        far2d_warps<R, OUT><<<(int)std::min<int64_t>((a.n + 3) / 4, (int64_t)nsm * 16), 128, 0, s>>>(a);
         return cudaSuccess;
     }
     const size_t sm = sizeof(double) * ((F2_Y * F2_S + 1 + F2_TAB + 1) & ~1) + sizeof(double2) * F2_TAB * (OUT == GF_OUT_HESSDIFF ? 2 : 1);
     cudaError_t e = cudaFuncSetAttribute(far2d<R, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    far2d<R, OUT><<<nsm, F2_THR, sm, s>>>(a);
+    far2d<R, OUT><<<nsm, F2_THR, sm, s>>>(a, lgmin);
     return cudaSuccess;
 }
 
