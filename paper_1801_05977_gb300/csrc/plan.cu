@@ -795,10 +795,13 @@ static gf_status eval_points(gf_plan_t p, const double *dev_xyz, int64_t n, int 
     const size_t off_buf = (sizeof(int) * ints + 255) / 256 * 256;
     size_t buf_bytes = slabs ? (size_t)slabcap * gf_out_entries(which) * p->elem : 0;
     // far targets by matrix products: from gf_far_product_min targets on, propagating indices
-    // within the one block of rows that the products give them (k < 7), no far-region grid
+    // within the one block of rows that the products give them (k < 7), no far-region grid.  A cell's
+    // fixed point is laid out for its largest weight, that of the tensor entries (up to about 1/k^2 times G_d's), and its
+    // digits reach 6 bits below a rounding of the plan's type: G_d beside them keeps its precision down to k = 0.2
     size_t mma_bytes = 0;
     int mma_cells = 0;
-    if (slabs && n >= gf_far_product_min(p->precision, p->nf, p->tr.c) && p->k < 7.0 && !p->fargrid && which != GF_OUT_LD)
+    if (slabs && n >= gf_far_product_min(p->precision, p->nf, p->tr.c) && p->k < 7.0 && !p->fargrid && which != GF_OUT_LD &&
+        !(which == GF_OUT_MAXWELL7 && p->k < 0.2))
         mma_bytes = gf_far_product_bytes(p->precision, n, p->nf == 1 ? 1 : gf_out_entries(which), &mma_cells);
     size_t off_mma = (off_buf + 2 * buf_bytes + 255) / 256 * 256;
     int *scratch = nullptr;
