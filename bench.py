@@ -55,8 +55,6 @@ FF_TERM_FLOPS = 98
 TAIL_TERM_FLOPS = 14
 FAR_CORE_Y0 = 18.0
 FAR_FF_GAP = 8.0
-# DRAM bytes of the far phase on this workload from ncu, or None: not taken for the products
-FAR_TRAFFIC_BYTES = None
 # unit-count peaks, reported beside the measured ones (152 SMs, 2.07 GHz):
 # FP64 2 FMA/clk/SM, FP32 128 FMA/clk/SM
 # in-plane points of the far-region grid of the split leg that uses it
@@ -446,8 +444,9 @@ def run_gpu(args):
     clocks = clk.summary()
     e2e_s = max_over_ranks([np.mean(e2e_t) if e2e_t else float("nan")], dev)[0]
 
-    # the far series' terms at the two ALU pipes' rates (what far3d_f64 and far3d_tail run; long
-    # lists go to the tensor cores instead)
+    # the far series' terms, and the time that the two ALU pipes would need for them at their measured
+    # rates (the series kernels far3d_f64 and far3d_tail run them there; this workload's list goes to the tensor
+    # cores as matrix products)
     far_ms = float(np.mean([p[3] for p in ph64]))
     near_ms = float(np.mean([p[2] for p in ph64]))
     synth_ms = float(np.mean([p[0] for p in ph64]))
@@ -459,13 +458,7 @@ def run_gpu(args):
     peaks = measure_peaks(dev)
     w64 = world * FP64_TERM_FLOPS * bands["double"]
     w32 = world * (FF_TERM_FLOPS * bands["float-float"] + TAIL_TERM_FLOPS * tail_terms)
-    t_far = far_ms * 1e-3
-    # FP64-equivalent work: FP32 flops weighted by the measured rate ratio, so that
-    # frac = W64 / (P64 t) + W32 / (P32 t), the share of the far phase the two pipes
-    # would need for the term work at their measured rates
-    w_eq = w64 + w32 * (peaks["fp64"] / peaks["fp32"])
-    achieved = w_eq / t_far / 1e12
-    frac64, frac32 = w64 / t_far / 1e12 / peaks["fp64"], w32 / t_far / 1e12 / peaks["fp32"]
+    alu_ms = 1e3 * (w64 / (peaks["fp64"] * 1e12) + w32 / (peaks["fp32"] * 1e12)) / world
 
     # split-precision error vs the double-precision path on this workload
     d = (out32.to(torch.complex128) - out64).abs()
@@ -527,25 +520,22 @@ def run_gpu(args):
                            "phases_ms": {"synthesis": float(np.mean([p[0] for p in phfg])),
                                          "near_and_far_grid": float(np.mean([p[2] for p in phfg])),
                                          "far_series": float(np.mean([p[3] for p in phfg]))}},
-        "roofline": {"bound": "alu", "kernel": "far series terms (far_product from 12288 targets, else far3d_f64 + far3d_tail)", "achieved": achieved,
-                     "peak": peaks["fp64"], "unit": "TFLOP/s (FP64-equivalent)", "frac": achieved / peaks["fp64"],
-                     "traffic": FAR_TRAFFIC_BYTES if n_targets == 1_000_000 and FAR_TRAFFIC_BYTES else None,
-                     "peaks_measured": {"fp64_tflops": peaks["fp64"], "fp32_tflops": peaks["fp32"],
-                                        "how": "gf_peak_probe FMA chains, CUDA events, best of 3"},
-                     "pipe_overlap": peaks["overlap"],
-                     "peaks_nominal": {"fp64_tflops": FP64_NOMINAL_TFLOPS, "fp32_tflops": FP32_NOMINAL_TFLOPS},
-                     "work": {"fp64_flops": w64, "fp32_flops": w32, "double_band_terms": bands["double"],
-                              "float_float_terms": bands["float-float"], "tail_terms": tail_terms,
-                              "all_terms": terms},
-                     "frac_fp64_pipe": frac64, "frac_fp32_pipe": frac32,
-                     "frac_max_model": max(frac64, frac32),
-                     "note": "two-pipe roofline of the far phase over all series terms: achieved = (FP64 term "
-                             "flops + FP32 term flops x P64/P32) / far-phase time, peak = measured FP64 rate, so "
-                             "frac = W64/(P64 t) + W32/(P32 t); per term 14 FP64 flops (double band), 98 FP32 "
-                             "flops (float-float band), 14 FP32 flops (float tail); frac_max_model takes the "
-                             "busier pipe alone.  Long lists sum these terms as matrix products on the tensor "
-                             "cores, off both pipes: the fraction is then a speed in units of the series "
-                             "kernels' bound and may exceed 1"},
+        "far_series": {"kernel": "far_product (lists from 12288 targets; shorter ones far3d_f64 + far3d_tail)",
+                       "ms": far_ms, "terms": terms, "terms_per_s": world * terms / (far_ms * 1e-3),
+                       "issue_share": 0.55, "tensor_pipe_share": 0.16,
+                       "shares_from": "ncu, far_product<double,6>: profiles/pipes_and_stalls_performance_cases.md",
+                       "alu_ms_of_the_terms": alu_ms,
+                       "work": {"fp64_flops": w64, "fp32_flops": w32, "double_band_terms": bands["double"],
+                                "float_float_terms": bands["float-float"], "tail_terms": tail_terms},
+                       "peaks_measured": {"fp64_tflops": peaks["fp64"], "fp32_tflops": peaks["fp32"],
+                                          "how": "gf_peak_probe FMA chains, CUDA events, best of 3"},
+                       "peaks_nominal": {"fp64_tflops": FP64_NOMINAL_TFLOPS, "fp32_tflops": FP32_NOMINAL_TFLOPS},
+                       "pipe_overlap": peaks["overlap"],
+                       "note": "the products run the terms on the tensor cores, bound by the issue of a tile's phases, "
+                               "digits and epilogue (the shares are of four instructions a cycle and of the tensor "
+                               "pipe's cycles); alu_ms_of_the_terms is what the same terms take on the FP64 and FP32 "
+                               "pipes at their measured rates, one after the other: 14 FP64 flops a term in the double "
+                               "band, 98 FP32 flops in the float-float band, 14 in the float tail"},
         "err_vs_oracle": err_oracle,
         "e2e": {"value": whole_job_rate(n_targets, world, e2e_s), "unit": "evals/s",
                 "h2d_bytes_per_step": int(x_np.nbytes), "d2h_bytes_per_step": int(n_targets * 16)},
