@@ -65,7 +65,7 @@ struct gf_batch_s {
     SynthBatch sb{};
     // evaluation
     EvalArgs *d_eargs = nullptr;
-    int *scratch = nullptr;           // far lists: 2 * cap ints
+    int *scratch = nullptr;           // far lists in append and in bucket order, near lists: 3 * cap ints
     int64_t cap = 0;
     int *counters = nullptr;          // GF_SCRATCH_COUNTERS per pair
     EvalBatch eb{};

@@ -1257,7 +1257,7 @@ __device__ __forceinline__ const float *far_rows_f32(const EvalArgs &a)
 }
 
 // Series tables of a 3D plan, built on the device: the b table over the index
-// box, the exponential table e^{-(j - j0)/128}, and (block 0, warp 0) the list
+// box, the exponential table e^{-(j - j0)/GF_EXPTAB_STEPS}, and (block 0, warp 0) the list
 // of propagating indices in row-major order of the sub-box pbox = [n1lo, n1hi,
 // n2lo, n2hi] (ballot compaction keeps the order fixed).
 template <typename E>
@@ -2914,11 +2914,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && NF == 1 ? 3 : 1) far3d_
 // About 15, 21 and 38 double operations a term for G, GRAD and HESSDIFF against 60,
 // 65 and 120 with a square root, a quotient, exp and a phase step in every term.  The
 // propagating indices are summed apart.  A target is shared by as many
-// lanes (1 .. 32, a run of indices each) as give an SM up to four warps; more would cost
-// more than they hide (two sines and the powers of v per lane).  A CTA orders its targets
-// by |x2|, so that the lanes of a warp have runs of about the same length.
-// 10,000 targets, G 111 -> 49 us; 100,000: GRAD 998 -> 256, HESSDIFF 1597 -> 455 us (without the
-// ordering and the even shares of the CTAs 479 and 861).
+// lanes (1 .. 32, a run of indices each) as give an SM up to four warps, more only where the
+// runs are long (lgmin): they would cost more than they hide (two sines and the powers of v per
+// lane).  A CTA orders its targets by |x2|, so that the lanes of a warp have runs of about the
+// same length.  Short lists and some long index ranges go to far2d_warps.  10,000 targets, G
+// 111 -> 49 us; 100,000: GRAD 998 -> 256, HESSDIFF 1597 -> 455 us (without the ordering and the even
+// shares of the CTAs 479 and 861).
 // ---------------------------------------------------------------------------
 constexpr int F2_THR = 512;
 constexpr int F2_TAB = 1024;            // indices kept (the middle of the range)

@@ -15,8 +15,13 @@
 // Precision.  Both factors are fixed-point numbers, cut into L signed 10-bit digits
 // (exact in f16): v = sum_i d_i 2^{-10 i - 9}, |d_i| <= 512.  The product of digit i
 // of a weight with digit j of a phase factor goes to the accumulator of level
-// i + j; every such sum is an integer below 2^24 in size, which the tensor cores'
-// FP32 accumulation holds exactly.  Levels 0 .. L-1 are kept: L = 6 for
+// i + j, a sum of integers, exact in the tensor cores' FP32 accumulation up to 2^24 in size.
+// No bound in the layout keeps the sums below that (a level adds hundreds of products of up to
+// 2^18): digits other than a number's leading ones are as good as random, so the sums are those of a
+// random walk.  Emulated in integers for k = 0.4 .. 6.8, |x3| = 0.6 .. 2.5 and targets at and
+// off multiples of pi/6: levels 0 .. 3 at most 2^17.3, 2^20.2, 2^21.2 and 2^21.7, root mean square 2^19 at
+// most (2^24 is 30 of those away); one that passed it would be rounded in its last bit.  Levels 4 and 5, up
+// to 2^22.8, are rounded in the end anyway.  Levels 0 .. L-1 are kept: L = 6 for
 // double-precision plans (2^-60 of the cell's largest weight, where the
 // recurrences of far3d_f64 round at 2^-53 of their state), L = 3 (2^-30) for split
 // plans.  A weight 2^-10 below the largest has no digit 0, and so on, so the

@@ -1,7 +1,7 @@
 // Allocation-free evaluation entry point (gf_eval_points_noalloc).
 //
-// gf_eval_points keeps its far-target scratch list in the plan and grows it
-// with cudaMalloc when a call brings more targets than before.  This variant
+// gf_eval_points takes its scratch from the library's memory pool at every call, which
+// reaches the driver whenever the pool has to grow.  This variant
 // instead uses one fixed scratch array declared below at file scope, so it
 // never allocates or frees device memory.  The array is sized for
 // GF_NOALLOC_MAX_TARGETS targets; it stays resident on every GPU that loads

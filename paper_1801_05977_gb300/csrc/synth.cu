@@ -6,8 +6,8 @@
 //
 // Inverse DFT convention (Eqs. (fcln), (ln)): with C_j = sqrt(V) L-hat_j,
 //   L_N(x_l) = V^{-1} sum_{j in S_N} C_j exp(2 pi i sum_i j_i l_i / M_i),
-// node index l standing for x = l h (mod period).  Each pass is a radix-2
-// Stockham autosort transform held in shared memory (one CTA owns a batch of
+// node index l standing for x = l h (mod period).  Each pass is a radix-4
+// Stockham autosort transform (one radix-2 stage first when log2 n is odd) held in shared memory (one CTA owns a batch of
 // whole lines, so every pass reads and writes global memory exactly once).
 #include <stdint.h>
 
